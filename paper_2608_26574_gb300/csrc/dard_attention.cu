@@ -27,11 +27,21 @@
 //   warps 4q .. 4q + 3  softmax and epilogue of tile q, one thread per query row;
 //   warp 8              TMA producer: both Q tiles, then K and V through 2 stages each;
 //   warp 9              TMEM allocator and S issuer: S_q(j) = Q_q K(j)^T (Q from shared
-//                       memory), once PV_q(j - 1) has read P_q(j - 1) out of S_q's columns;
-//   warp 10             PV issuer: O_q += P_q(j) V(j), each 64-key half as soon as that half
-//                       of P_q(j) is stored.
-//   TMEM: S_0, S_1 [0, 256) with P_q(j) written over the first 64 columns of S_q(j),
-//   O_0, O_1 [256, 256 + 2D).
+//                       memory), once the softmax has read the scores before it out of
+//                       the S buffer into registers;
+//   warp 10             PV issuer: O_q += P_q(j) V(j), once P_q(j) is stored and S_q(j + 1)
+//                       has been issued.
+//   TMEM: the S buffer [0, 128), P_0, P_1 [128, 256), O_0, O_1 [256, 256 + 2D); at D = 64 a
+//   second S buffer [384, 512).
+//   Bound: the tensor pipe. A pair of tiles takes 2064 cycles of products per key tile
+//   (each M128 N128 K16 product 64.5, whatever the operand's form) and about 2300 in the
+//   steady state. What that took, on one layer of 28 / 4 heads and 5184 rows (308 us and
+//   3460 cycles before, 217 us after): P in columns of its own, so that S_q(j + 1) waits for
+//   a register read instead of for PV_q(j) (297 us); issue by an elected lane of a converged
+//   warp (280 us; in a one-lane branch an MMA took 100 cycles to issue); PV_q(j) behind
+//   S_q(j + 1) in the pipe, since the one S buffer's turnaround is the critical path and the
+//   pipe runs two threads' products interleaved (231 us); no maximum and no mask arithmetic on
+//   the common tile (217 us).
 // Both keep a per-row running maximum and rescale O in TMEM only when the maximum grows by
 // more than a factor 2^8 (the exponentials stay bounded by 2^8 otherwise).
 // fp32 path: attn_simt (dard_attention_simt.cu), CUDA cores, the same mask logic.
@@ -51,6 +61,7 @@ constexpr int kTc2Threads = 384;  // attn_tc2: 2 x 4 softmax warps, TMA producer
 
 constexpr int kQT = 2;   // query tiles per CTA (the same sequence and head)
 constexpr int kNK = 2;   // TMA stages for K
+constexpr int kPvGo = 4;  // slots of the S-before-PV hand-off
 constexpr int kNV = 2;   // TMA stages for V
 constexpr int kWProd = 2 * kQT * 2;  // warp 8: TMA producer
 constexpr int kWMma = kWProd + 1;    // warp 9: TMEM allocator and S issuer
@@ -59,7 +70,7 @@ constexpr int kWPv = kWProd + 2;     // warp 10: PV issuer
 // warpgroup of warps 8-11 (producer, issuers, spare) drops to 56 and the two softmax
 // warpgroups rise to 224, so that a thread holds its row's 128 scores at once:
 // 128 x 56 + 256 x 224 = 384 x 168.
-constexpr uint32_t kTc2LaunchRegs = 168, kTc2SideRegs = 56, kTc2SoftmaxRegs = 224;
+constexpr uint32_t kTc2LaunchRegs = 168, kTc2SideRegs = 40, kTc2SoftmaxRegs = 232;
 static_assert(128 * kTc2SideRegs + 256 * kTc2SoftmaxRegs == kTc2Threads * kTc2LaunchRegs,
               "the register shares must add up to the launch's registers");
 static_assert(kTc2Threads * kTc2LaunchRegs <= 65536, "one CTA per SM");
@@ -483,22 +494,17 @@ __global__ void __launch_bounds__(kTc1Threads, 1)
 }
 
 
-// One query row's 128-key S tile out of TMEM (columns tS .. tS + 127 of its lane) into
-// registers, with the visibility bits applied (kMasked; vis0: keys 0-63, vis1: 64-127, a
-// hidden key becomes -inf); returns the row maximum. One wait for the four loads.
-template <bool kMasked>
-__device__ __forceinline__ float tile_row_load(uint32_t tS, uint64_t vis0, uint64_t vis1,
-                                               uint32_t (&sv)[128]) {
+// The visibility bits applied to a row's 128 scores (vis0: keys 0-63, vis1: 64-127): a hidden
+// key becomes -inf.
+__device__ __forceinline__ void mask_row(uint64_t vis0, uint64_t vis1, uint32_t (&sv)[128]) {
 #pragma unroll
-  for (int c = 0; c < 4; ++c) tmem_ld32(tS + 32 * c, *reinterpret_cast<uint32_t(*)[32]>(sv + 32 * c));
-  tmem_wait_ld();
-  if (kMasked) {
-#pragma unroll
-    for (int k = 0; k < 128; ++k) {
-      const uint64_t vis = k < 64 ? vis0 : vis1;
-      sv[k] = ((vis >> (k & 63)) & 1ull) ? sv[k] : 0xff800000u;  // -inf
-    }
+  for (int k = 0; k < 128; ++k) {
+    const uint64_t vis = k < 64 ? vis0 : vis1;
+    sv[k] = ((vis >> (k & 63)) & 1ull) ? sv[k] : 0xff800000u;  // -inf
   }
+}
+
+__device__ __forceinline__ float tile_row_max(const uint32_t (&sv)[128]) {
   float mx[8];
 #pragma unroll
   for (int e = 0; e < 8; ++e)
@@ -513,29 +519,25 @@ __device__ __forceinline__ float tile_row_load(uint32_t tS, uint64_t vis0, uint6
   return fmaxf(fmax3(mx[0], mx[1], mx[2]), fmax3(fmax3(mx[3], mx[4], mx[5]), mx[6], mx[7]));
 }
 
-// P = 2^(s * sl - mL) for keys 64 hh .. 64 hh + 63 of the row's 128 scores held in
-// registers, stored as bf16 pairs over columns tS + 32 hh .. tS + 32 hh + 31 (in the first
-// half of the S tile's columns); the stored (rounded) values are summed into acc (four packed
-// partial sums), so that the output is a convex combination of V rows with exactly the
-// weights the PV product uses.
-template <int hh>
-__device__ __forceinline__ void tile_row_exp(uint32_t tS, const uint32_t (&sv)[128],
-                                             uint64_t sl2, uint64_t nmL2, uint64_t (&acc)[4]) {
-  {
-    uint32_t pk[32];
+// P = 2^(s * sl - mL) of the row's 128 scores as bf16 pairs, and their sum: of the rounded
+// values, so that the output is a convex combination of V rows with exactly the weights the
+// PV product uses.
+__device__ __forceinline__ float tile_row_exp(const uint32_t (&sv)[128], uint64_t sl2,
+                                              uint64_t nmL2, uint32_t (&pk)[64]) {
+  uint64_t acc[4] = {0, 0, 0, 0};  // bit pattern 0 = +0.0f
 #pragma unroll
-    for (int e = 0; e < 32; ++e) {
-      float x0, x1;
-      f2_unpack(f2_fma(f2_pack(__uint_as_float(sv[64 * hh + 2 * e]),
-                               __uint_as_float(sv[64 * hh + 2 * e + 1])), sl2, nmL2), x0, x1);
-      pk[e] = pack_bf16x2(ex2_approx(x0), ex2_approx(x1));
-      // the row sum adds the rounded weights the PV product multiplies with (unpacked by
-      // shift and mask into a packed pair: faster here than two mixed-precision adds)
-      acc[e & 3] = f2_add(acc[e & 3], f2_pack(__uint_as_float(pk[e] << 16),
-                                              __uint_as_float(pk[e] & 0xffff0000u)));
-    }
-    tmem_st32(tS + 32 * hh, pk);
+  for (int e = 0; e < 64; ++e) {
+    float x0, x1;
+    f2_unpack(f2_fma(f2_pack(__uint_as_float(sv[2 * e]), __uint_as_float(sv[2 * e + 1])), sl2,
+                     nmL2), x0, x1);
+    pk[e] = pack_bf16x2(ex2_approx(x0), ex2_approx(x1));
+    acc[e & 3] = f2_add(acc[e & 3], f2_pack(__uint_as_float(pk[e] << 16),
+                                            __uint_as_float(pk[e] & 0xffff0000u)));
   }
+  float a0, a1, b0, b1;
+  f2_unpack(f2_add(acc[0], acc[1]), a0, a1);
+  f2_unpack(f2_add(acc[2], acc[3]), b0, b1);
+  return (a0 + a1) + (b0 + b1);
 }
 
 // Barrier protocol. Every barrier completes one phase per use; use u waits for parity
@@ -546,8 +548,15 @@ struct __align__(16) Tc2Ctl {
   uint64_t q_full[kQT];  // query tile q landed
   uint64_t q_rot[kQT];   // RoPE: the softmax warps of tile q rotated it in shared memory
   uint64_t k_full[kNK], k_empty[kNK], v_full[kNV], v_empty[kNV];
-  uint64_t s_full[kQT];   // S_q(j) landed in TMEM
-  uint64_t p_half[kQT][2];  // the softmax of tile q stored keys 64 h .. 64 h + 63 of P_q(j)
+  uint64_t s_full[kQT];   // S_q(j) landed in TMEM: per tile with two tiles, else per buffer
+  uint64_t s_free[kQT];   // per buffer: the softmax read the scores into registers
+  uint64_t p_full[kQT];   // the softmax of tile q stored P_q(j)
+  // S_q(j + 1) has been issued: PV_q(j) may follow it into the pipe. A ring of kPvGo, since
+  // S runs ahead: S_q(j + 4) is only issued once the softmax has read S_q(j + 2) (its buffer,
+  // or one before it in turn), so has stored P_q(j + 1), which waits for PV_q(j): the
+  // issuer of PV has taken phase j of its slot before phase j + 4 completes (and before
+  // j + 3: three slots would do).
+  uint64_t pv_go[kQT][kPvGo];
   uint64_t pv_done[kQT];  // PV_q(j) completed: S_q's columns may take S_q(j + 1)
   uint64_t o_full[kQT];   // the last PV_q completed
   uint64_t drained;       // every product both issuers launched has completed (two commits)
@@ -577,6 +586,7 @@ __global__ void __launch_bounds__(kTc2Threads, 1)
   constexpr int kSub = D / 64;                   // 128-byte (64 x bf16) column blocks
   constexpr uint32_t kKSub = kTN * 128;          // one 128-row x 128-byte swizzled block
   constexpr uint32_t kTileBytes = kSub * kKSub;  // one 128-row tile of Q, K or V
+  constexpr int kNX = D == 64 ? 2 : 1;           // S buffers in TMEM
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -634,8 +644,9 @@ __global__ void __launch_bounds__(kTc2Threads, 1)
     }
     for (int q = 0; q < kQT; ++q) {
       mbar_init(&ctl.s_full[q], 1);
-      mbar_init(&ctl.p_half[q][0], 4);
-      mbar_init(&ctl.p_half[q][1], 4);
+      mbar_init(&ctl.s_free[q], 4);
+      mbar_init(&ctl.p_full[q], 4);
+      for (int b = 0; b < kPvGo; ++b) mbar_init(&ctl.pv_go[q][b], 1);
       mbar_init(&ctl.pv_done[q], 1);
       mbar_init(&ctl.o_full[q], 1);
     }
@@ -659,10 +670,12 @@ __global__ void __launch_bounds__(kTc2Threads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  // TMEM columns: S_q / P_q [128 q, 128 q + 128) (P_q(j) as bf16 pairs over the first 64),
-  // O_q [256 + D q, 256 + D q + D)
-  const uint32_t tS0 = ctl.tmem_base;
+  // TMEM columns: the first S buffer [0, 128), P_q [128 + 64 q, 192 + 64 q) (bf16 pairs),
+  // O_q [256 + D q, 256 + D q + D), at D = 64 a second S buffer [384, 512)
+  const uint32_t tX0 = ctl.tmem_base;
+  const uint32_t tP0 = ctl.tmem_base + kTN;
   const uint32_t tO0 = ctl.tmem_base + kQT * kTN;
+  auto s_buf = [&](int b) { return tX0 + (b != 0 ? 384u : 0u); };
   volatile int32_t* abort_flag = &ctl.abort;
 
   // The register split: each branch below starts with its warpgroup's setmaxnreg (warps 8-11
@@ -719,69 +732,73 @@ __global__ void __launch_bounds__(kTc2Threads, 1)
   } else if (warp == kWMma) {
     // ------------------------------------------------------------ S issuer
     reg_dealloc<kTc2SideRegs>();
-    // S_q(j) = Q_q K(j)^T once K(j) has landed and, for j > 0, PV_q(j - 1) has completed
-    // (S_q(j) overwrites the P_q(j - 1) that PV_q(j - 1) reads). The PV products come from
-    // a second issuer thread: one thread issuing both kinds of product in turn leaves the
-    // tensor pipe at about two thirds of its rate on this GPU.
-    if (lane == 0) {
-      constexpr uint32_t kIdS = idesc_bf16_f32(kBM, kTN, 0, 0);
-      const uint32_t aq = smem_u32(sQ), ak = smem_u32(sK);
-      bool ok = true;
-      for (int j = 0; j < n_kt && ok && !*abort_flag; ++j) {
-        ok = mbar_wait(&ctl.k_full[j % kNK], (j / kNK) & 1, wlim);
-        for (int q = 0; q < nq && ok; ++q) {
-          if (j == 0) ok = mbar_wait(kRope ? &ctl.q_rot[q] : &ctl.q_full[q], 0, wlim);
-          else ok = mbar_wait(&ctl.pv_done[q], (j - 1) & 1, wlim);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t qaddr = aq + q * kTileBytes, kaddr = ak + (j % kNK) * kTileBytes;
+    // S_q(j) = Q_q K(j)^T once K(j) has landed and the softmax has read the scores that the
+    // buffer held out of it. The whole warp runs the loop and an elected lane issues:
+    // descriptors and addresses then stay in uniform registers, where the instruction wants
+    // them (in a one-lane branch each MMA took about 100 cycles to issue, more than the 64
+    // that it runs). The PV products come from a second warp, whose waits between products
+    // then hide behind this one's products and the other way round.
+    constexpr uint32_t kIdS = idesc_bf16_f32(kBM, kTN, 0, 0);
+    const uint64_t dq = smem_desc_sw128(smem_u32(sQ), 16, 1024);
+    const uint64_t dk = smem_desc_sw128(smem_u32(sK), 16, 1024);
+    bool ok = true;
+    for (int j = 0; j < n_kt && ok; ++j) {
+      ok = warp_wait(&ctl.k_full[j % kNK], (j / kNK) & 1, wlim);
+      const uint64_t db = dk + (j % kNK) * (kTileBytes >> 4);
+      for (int q = 0; q < nq && ok; ++q) {
+        const int u = j * nq + q, xb = u % kNX;  // the u-th S product of the CTA, its buffer
+        if (j == 0) ok = warp_wait(kRope ? &ctl.q_rot[q] : &ctl.q_full[q], 0, wlim);
+        if (ok && u >= kNX) ok = warp_wait(&ctl.s_free[xb], (u / kNX - 1) & 1, wlim);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t da = dq + q * (kTileBytes >> 4);
+        const uint32_t td = s_buf(xb);
+        if (elect_one()) {
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks) {
-            const uint32_t off = (ks >> 2) * kKSub + (ks & 3) * 32;
-            mma_ss(tS0 + q * kTN, smem_desc_sw128(qaddr + off, 16, 1024),
-                   smem_desc_sw128(kaddr + off, 16, 1024), kIdS, ks > 0);
+            const uint32_t off = ((ks >> 2) * kKSub + (ks & 3) * 32) >> 4;
+            mma_ss(td, da + off, db + off, kIdS, ks > 0);
           }
-          mma_commit(&ctl.s_full[q]);
+          mma_commit(&ctl.s_full[nq == 1 ? xb : q]);
+          if (q == nq - 1) mma_commit(&ctl.k_empty[j % kNK]);
+          if (j > 0) mbar_arrive(&ctl.pv_go[q][(j - 1) % kPvGo]);  // PV_q(j - 1) may follow
         }
-        if (ok) mma_commit(&ctl.k_empty[j % kNK]);
+        __syncwarp();
       }
-      if (!ok) flag_timeout(p, ctl);
-      mma_commit(&ctl.drained);  // completes once every S product this thread issued has
     }
+    if (!ok && lane == 0) flag_timeout(p, ctl);
+    if (elect_one()) mma_commit(&ctl.drained);  // completes once every S product issued has
+    __syncwarp();
   } else if (warp == kWPv) {
     // ------------------------------------------------------------ PV issuer
     reg_dealloc<kTc2SideRegs>();
-    // O_q += P_q(j) V(j) once V(j) has landed, in two halves of 64 keys: each as soon as
-    // the softmax of tile q has stored that half of P_q(j), so that the first half's
-    // products run while the softmax computes the second.
-    if (lane == 0) {
-      constexpr uint32_t kIdO = idesc_bf16_f32(kBM, D, 0, 1);
-      const uint32_t av = smem_u32(sV);
-      bool ok = true;
-      for (int j = 0; j < n_kt && ok && !*abort_flag; ++j) {
-        ok = mbar_wait(&ctl.v_full[j % kNV], (j / kNV) & 1, wlim);
-        for (int q = 0; q < nq && ok; ++q) {
-          const uint32_t vaddr = av + (j % kNV) * kTileBytes;
+    // O_q += P_q(j) V(j) once V(j) has landed and the softmax of tile q has stored P_q(j).
+    constexpr uint32_t kIdO = idesc_bf16_f32(kBM, D, 0, 1);
+    const uint64_t dv = smem_desc_sw128(smem_u32(sV), kKSub, 1024);
+    bool ok = true;
+    for (int j = 0; j < n_kt && ok; ++j) {
+      ok = warp_wait(&ctl.v_full[j % kNV], (j / kNV) & 1, wlim);
+      const uint64_t db = dv + (j % kNV) * (kTileBytes >> 4);
+      for (int q = 0; q < nq && ok; ++q) {
+        const uint32_t td = tO0 + q * D, ta = tP0 + q * 64;
+        ok = warp_wait(&ctl.p_full[q], j & 1, wlim) &&
+             (j + 1 == n_kt || warp_wait(&ctl.pv_go[q][j % kPvGo], (j / kPvGo) & 1, wlim));
+        if (!ok) break;
+        tc_fence_after();
+        if (elect_one()) {
 #pragma unroll
-          for (int hh = 0; hh < 2; ++hh) {
-            ok = ok && mbar_wait(&ctl.p_half[q][hh], j & 1, wlim);
-            if (!ok) break;
-            tc_fence_after();
-#pragma unroll
-            for (int ks = 4 * hh; ks < 4 * hh + 4; ++ks)
-              mma_ts(tO0 + q * D, tS0 + q * kTN + ks * 8,
-                     smem_desc_sw128(vaddr + ks * 2048, kKSub, 1024), kIdO,
-                     (j > 0 || ks > 0) ? 1u : 0u);
-          }
-          if (!ok) break;
+          for (int ks = 0; ks < kTN / 16; ++ks)
+            mma_ts(td, ta + ks * 8, db + ks * (2048 >> 4), kIdO, (j > 0 || ks > 0) ? 1u : 0u);
           mma_commit(&ctl.pv_done[q]);
           if (j == n_kt - 1) mma_commit(&ctl.o_full[q]);
+          if (q == nq - 1) mma_commit(&ctl.v_empty[j % kNV]);
         }
-        if (ok) mma_commit(&ctl.v_empty[j % kNV]);
+        __syncwarp();
       }
-      if (!ok) flag_timeout(p, ctl);
-      mma_commit(&ctl.drained);  // completes once every PV product this thread issued has
     }
+    if (!ok && lane == 0) flag_timeout(p, ctl);
+    if (elect_one()) mma_commit(&ctl.drained);  // completes once every PV product issued has
+    __syncwarp();
   } else if (warp < kWProd) {
     // ------------------------------------------------------------ softmax + epilogue
     // Warps 4q .. 4q + 3 own query tile q; thread t = query row t of the tile (TMEM lane t).
@@ -789,7 +806,7 @@ __global__ void __launch_bounds__(kTc2Threads, 1)
     const int q = warp >> 2, quarter = warp & 3;
     const int t = quarter * 32 + lane;
     const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
-    const uint32_t tS = tS0 + q * kTN, tO = tO0 + q * D;
+    const uint32_t tP = tP0 + q * 64, tO = tO0 + q * D;
     if (warp < 4) publish_block_info(p, sd, ctl.bi, bf, pr == 0 && h == 0);
     softmax_bar_sync();
     const int r = sd.q_start + (qt0 + q) * kBM + t;  // sequence-relative query row
@@ -810,28 +827,64 @@ __global__ void __launch_bounds__(kTc2Threads, 1)
     const float sl = p.scale_log2;
     float m_run = -INFINITY, l_run = 0.f;
     bool ok = active;
+    // the key tiles that need the mask (tile_needs_mask): those of the block, [jb0, jb1), and
+    // those from jm on
+    const int jb0 = sd.b0 / kTN, jb1 = sd.blen > 0 ? (sd.b0 + sd.blen + kTN - 1) / kTN : 0;
+    const int jm = sd.n_orig / kTN;
     for (int j = 0; j < n_kt && ok; ++j) {
-      const bool masked = tile_needs_mask(sd, j * kTN);
-      const uint64_t vis0 = masked ? vis64(sd, j * kTN, rm) : ~0ull;
-      const uint64_t vis1 = masked ? vis64(sd, j * kTN + 64, rm) : ~0ull;
-      ok = !*abort_flag && mbar_wait(&ctl.s_full[q], j & 1, wlim);
+      const int xb = (j * nq + q) % kNX;  // the buffer of S_q(j)
+      ok = (nq == 1 ? mbar_wait(&ctl.s_full[xb], (j / kNX) & 1, wlim)
+                    : mbar_wait(&ctl.s_full[q], j & 1, wlim));
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       tc_fence_after();
       // the tile's 128 scores of this row in registers, and their maximum
       uint32_t sv[128];
-      const float mt = masked ? tile_row_load<true>(tS + lane_off, vis0, vis1, sv)
-                              : tile_row_load<false>(tS + lane_off, vis0, vis1, sv);
-      // Raise the reference maximum on the first finite value, or when the tile maximum
-      // exceeds it by more than 2^kRescaleLog2 in probability; only then is O rescaled.
-      float m_new = m_run;
-      if (m_run == -INFINITY) m_new = mt;
-      else if ((mt - m_run) * sl > kRescaleLog2) m_new = mt;
-      const bool rescale = (m_new != m_run) && (m_run != -INFINITY);
-      const float alpha = rescale ? ex2_approx((m_run - m_new) * sl) : 1.f;
-      const float mL = (m_new == -INFINITY) ? 0.f : m_new * sl;
-      // PV_q(j - 1) completed before S_q(j) was issued: O_q may be rescaled right away.
-      if (__any_sync(0xffffffffu, rescale)) {
 #pragma unroll
+      for (int c = 0; c < 4; ++c)
+        tmem_ld32(s_buf(xb) + lane_off + 32 * c, *reinterpret_cast<uint32_t(*)[32]>(sv + 32 * c));
+      tmem_wait_ld();
+      // the scores are in registers: the buffer may take the next S product
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&ctl.s_free[xb]);
+      if (j >= jm || (j >= jb0 && j < jb1))
+        mask_row(vis64(sd, j * kTN, rm), vis64(sd, j * kTN + 64, rm), sv);
+      // P_q(j) replaces P_q(j - 1), and O_q may be rescaled, once PV_q(j - 1) has completed:
+      // asked early, it seldom has to be waited for below
+      const bool pv_ok = j == 0 || mbar_try_wait(&ctl.pv_done[q], (j - 1) & 1);
+      // The reference maximum: that of the first tile with a finite score.
+      if (__any_sync(0xffffffffu, m_run == -INFINITY)) {
+        const float mt = tile_row_max(sv);
+        if (m_run == -INFINITY) m_run = mt;
+      }
+      // The tile's weights against the reference so far. Their sum stays below
+      // 2^kRescaleLog2 unless the tile's maximum exceeds the reference by more than that in
+      // probability; only then is the maximum formed, the reference raised to it, the
+      // weights computed again and O rescaled.
+      const uint64_t sl2 = f2_pack(sl, sl);
+      const float mL = m_run == -INFINITY ? 0.f : m_run * sl;
+      uint64_t nmL2 = f2_pack(-mL, -mL);
+      uint32_t pk[64];
+      float ls = tile_row_exp(sv, sl2, nmL2, pk);
+      float alpha = 1.f;
+      bool rescale = false;
+      if (__any_sync(0xffffffffu, !(ls < kRescaleMax))) {
+        const float mt = tile_row_max(sv);
+        if ((mt - m_run) * sl > kRescaleLog2) {
+          rescale = true;
+          alpha = ex2_approx((m_run - mt) * sl);
+          m_run = mt;
+          nmL2 = f2_pack(-m_run * sl, -m_run * sl);
+        }
+        ls = tile_row_exp(sv, sl2, nmL2, pk);
+      }
+      if (!__all_sync(0xffffffffu, pv_ok)) {
+        ok = mbar_wait(&ctl.pv_done[q], (j - 1) & 1, wlim);
+        if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+      }
+      tc_fence_after();
+      if (__any_sync(0xffffffffu, rescale)) {
+#pragma unroll 1
         for (int c = 0; c < D / 32; ++c) {
           uint32_t o[32];
           tmem_ld32(tO + lane_off + 32 * c, o);
@@ -841,25 +894,14 @@ __global__ void __launch_bounds__(kTc2Threads, 1)
           tmem_st32(tO + lane_off + 32 * c, o);
         }
       }
-      // P over the first 64 columns of S_q(j), and the row sum
-      const uint64_t sl2 = f2_pack(sl, sl), nmL2 = f2_pack(-mL, -mL);
-      uint64_t acc[4] = {0, 0, 0, 0};  // bit pattern 0 = +0.0f
-      // the first half of P, handed to the PV issuer before the second is computed
-      tile_row_exp<0>(tS + lane_off, sv, sl2, nmL2, acc);
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        tmem_st32(tP + lane_off + 32 * c, *reinterpret_cast<const uint32_t(*)[32]>(pk + 32 * c));
+      l_run = fmaf(l_run, alpha, ls);
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&ctl.p_half[q][0]);
-      tile_row_exp<1>(tS + lane_off, sv, sl2, nmL2, acc);
-      float a0, a1, b0, b1;
-      f2_unpack(f2_add(acc[0], acc[1]), a0, a1);
-      f2_unpack(f2_add(acc[2], acc[3]), b0, b1);
-      l_run = l_run * alpha + ((a0 + a1) + (b0 + b1));
-      m_run = m_new;
-      tmem_wait_st();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&ctl.p_half[q][1]);
+      if (lane == 0) mbar_arrive(&ctl.p_full[q]);
     }
     if (active) {
       if (ok) ok = mbar_wait(&ctl.o_full[q], 0, wlim);

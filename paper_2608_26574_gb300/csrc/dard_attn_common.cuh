@@ -23,6 +23,7 @@ namespace {
 constexpr int kBM = 128;  // query rows per CTA
 constexpr uint32_t kTmemCols = 512;  // every TMEM column of the SM
 constexpr float kRescaleLog2 = 8.0f;
+constexpr float kRescaleMax = 256.0f;  // 2^kRescaleLog2
 
 // Per-CTA copy of the current block: states, confidences, the shadow maps, and the same
 // facts as bit words over block positions (word w = positions 32w .. 32w + 31).
