@@ -233,8 +233,8 @@ class AttentionCall:
 
     def kernel(self, q, k, v, o) -> int:
         """The kernel a call on these tensors launches, without launching it: 1 or 2 (the
-        tensor-core kernel with one or two query tiles per CTA), 4 (the CTA-pair kernel),
-        3 (fp32 CUDA cores), 0 (no query rows)."""
+        tensor-core kernel over single query tiles or pairs of a head's), 4 (the CTA-pair
+        kernel), 3 (fp32 CUDA cores), 0 (no query rows)."""
         self._bind(q, k, v, o, k if self.rope else None)
         out = ctypes.c_int32(-1)
         _check(lib().dard_attention_kernel(self._ref, ctypes.byref(out)), "dard_attention_kernel")

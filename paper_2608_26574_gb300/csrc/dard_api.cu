@@ -287,10 +287,11 @@ dard_status dard_attention_plan(const dard_attn_args* a, dard_attn_plan* plan) {
     plan->ctas = static_cast<int64_t>(p.total_work) * kSimtCtasPerTile;
     return DARD_OK;
   }
-  plan->ctas = plan->kernel == 1 ? p.total_work
-             : plan->kernel == 2 ? p.total_pairs
-                                 : 2ll * pair_clusters_for(p);
-  // rows handled together: one query tile (kernel 1), or two (kernels 2 and 4)
+  plan->ctas = plan->kernel == 4 ? 2ll * pair_clusters_for(p)
+             : p.persist         ? persist_ctas(p)
+             : plan->kernel == 1 ? p.total_work
+                                 : p.total_pairs;
+  // rows with one range of key tiles: a query tile (kernel 1), or two (kernels 2 and 4)
   const int unit = plan->kernel == 1 ? kKeyTile : 2 * kKeyTile;
   for (int s = 0; s < p.num_seqs; ++s) {
     const SeqDesc& sd = p.seq[s];

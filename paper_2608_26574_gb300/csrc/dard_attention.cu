@@ -9,7 +9,8 @@
 // shadow keys or the ragged end of the sequence.
 //
 // bf16 paths (tcgen05 MMAs with fp32 accumulators in TMEM, K/V tiles of 128 keys by TMA),
-// one CTA per SM, chosen per call by a cost model (launch_tc):
+// one CTA per SM, chosen per call by a cost model (choose_tc); launches of more than one wave
+// run attn_persist (dard_attention_persist.cu) instead:
 //
 // attn_tc1: 128 query rows of one (sequence, head); 11 warps:
 //   warps 0-7  softmax and epilogue: warps w and w + 4 share TMEM lane quarter w (query
@@ -965,43 +966,57 @@ __global__ void __launch_bounds__(kTc2Threads, 1)
 
 // ---------------------------------------------------------------- host side
 
-// Which tensor-core kernel: a cost model in SM cycles, fitted (least squares on the log of
-// the time) to CUDA-graph timings of both kernels on the full and prefix-cached variants
-// of four workload shapes on GB300 (within 6 % of each of the 16 timings). attn_tc1 costs
-// about 14250 + 1500 kt cycles per 128-row query tile (kt = tiles of 128 keys); attn_tc2
-// about 11900 + 3460 kt per pair of tiles and 32300 + 600 kt for a lone last tile (its
-// chain is latency-bound, much like a pair's). Work spreads over the SMs one CTA each: a
-// launch with no more CTAs than SMs takes its longest CTA, a larger one about total / SMs
-// plus half a CTA of tail. attn_tc2 wins on every full workload (8B layer: one wave instead
-// of 1.5, and its per-tile cost now below two of attn_tc1's), attn_tc1 on small query counts
-// (the 8B prefix-cached step); where the model errs (the GQA pair) the two differ by 1.5 %.
+// How query tiles make work items (dard_attention_kernel's 1 and 2) and which kernel runs
+// them, by a cost model in SM cycles fitted to CUDA-graph timings on GB300 (kt = tiles of 128
+// keys).
+//   1, at most one tile per SM: attn_tc1, about 14250 + 1500 kt;
+//   2, at most one pair of a head's tiles per SM: attn_tc2, about 14700 + 2300 kt (a lone
+//      last tile 14000 + 1700 kt);
+//   more than that: attn_persist over items of any two consecutive (tile, head) units of a K/V
+//      head's group (1) or of pairs of a head's tiles (2): 7000 + 2300 kt an item (a lone
+//      tile 7000 + 2000 kt) spread over the SMs, plus half an item of tail and 12000 to start.
+// Measured, us (8B layer, its prefix-cached variant, GQA sequence, its variant, ragged batch):
+// attn_tc1 22.8, 12.4, 301, 76, 1168; attn_tc2 15.4, 14.6, 217, 54, 811; attn_persist 17.7,
+// 14.7, 221, 58, 759. Equal costs go to 2: the two ways differ only where a group of heads or
+// an odd tile count lets 1 fill items that 2 leaves half empty, or where single tiles spread
+// over more SMs.
 struct TcEstimate {
   double total = 0, longest = 0;
-  long long ctas = 0;
+  long long items = 0;
   void add(long long n, double cost) {
     if (n <= 0) return;
     total += static_cast<double>(n) * cost;
     longest = std::max(longest, cost);
-    ctas += n;
+    items += n;
   }
-  double cycles(int sms) const {
-    return ctas <= sms ? longest : total / sms + 0.5 * longest;
+  double persistent(int sms) const {
+    return 12000.0 + (items <= sms ? longest : total / sms + 0.5 * longest);
   }
 };
 
-bool prefer_tc2(const AttnParams& p, int sms) {
-  TcEstimate one, two;
+// 1 or 2 (`forced`, or the cheaper one), with whether attn_persist runs it.
+int choose_tc(const AttnParams& p, int sms, int forced, bool* persist) {
+  TcEstimate tiles, pairs, group_items, pair_items;
+  const long long per_group = p.hq / p.hkv;
   for (int s = 0; s < p.num_seqs; ++s) {
     const SeqDesc& sd = p.seq[s];
     const double kt = (sd.n_orig + sd.slen + kTN - 1) / kTN;
-    const long long tiles = sd.n_qtiles, heads = p.hq;
-    one.add(tiles * heads, 14250.0 + 1500.0 * kt);
-    two.add((tiles / 2) * heads, 11900.0 + 3460.0 * kt);
-    two.add((tiles % 2) * heads, 32300.0 + 600.0 * kt);
+    const long long n = sd.n_qtiles, units = n * per_group;
+    tiles.add(n * p.hq, 14250.0 + 1500.0 * kt);
+    pairs.add(n / 2 * p.hq, 14700.0 + 2300.0 * kt);
+    pairs.add(n % 2 * p.hq, 14000.0 + 1700.0 * kt);
+    group_items.add(units / 2 * p.hkv, 7000.0 + 2300.0 * kt);
+    group_items.add(units % 2 * p.hkv, 7000.0 + 2000.0 * kt);
+    pair_items.add(n / 2 * p.hq, 7000.0 + 2300.0 * kt);
+    pair_items.add(n % 2 * p.hq, 7000.0 + 2000.0 * kt);
   }
-  return two.cycles(sms) < one.cycles(sms);
+  const bool wave1 = tiles.items <= sms, wave2 = pairs.items <= sms;
+  const double c1 = wave1 ? tiles.longest : group_items.persistent(sms);
+  const double c2 = wave2 ? pairs.longest : pair_items.persistent(sms);
+  const int kernel = forced != 0 ? forced : c2 <= c1 ? 2 : 1;
+  *persist = kernel == 1 ? !wave1 : !wave2;
+  return kernel;
 }
-
 
 // attn_tc2's register split assumes a launch allocation of kTc2LaunchRegs per thread; with
 // any other, setmaxnreg.inc would wait for registers that never come. A build that allocated
@@ -1048,14 +1063,17 @@ cudaError_t launch_tc(const AttnParams& p, int kernel, cudaStream_t stream) {
 
 }  // namespace
 
-int attention_kernel_choice(const dard_attn_args& a, const AttnParams& p) {
+int attention_kernel_choice(const dard_attn_args& a, AttnParams& p) {
   if (a.dtype == DARD_F32) return 3;
-  // DARD_ATTN_TC=1 or 2 forces one kernel (tests and tuning); anything else: the model
+  // DARD_ATTN_TC=1 or 2 forces one way (tests and tuning); anything else: the model
   const char* force = std::getenv("DARD_ATTN_TC");
   const int forced = force ? std::atoi(force) : 0;
-  if (forced == 1 || forced == 2) return forced;
-  if (forced == 4) return a.head_dim == 128 ? 4 : (prefer_tc2(p, sm_count()) ? 2 : 1);
-  return prefer_tc2(p, sm_count()) ? 2 : 1;
+  if (forced == 4 && a.head_dim == 128) return 4;
+  bool persist;
+  const int kernel = choose_tc(p, sm_count(), forced == 1 || forced == 2 ? forced : 0, &persist);
+  p.persist = persist;
+  if (persist) plan_items(p, kernel == 1);
+  return kernel;
 }
 
 dard_status launch_attention(const dard_attn_args& a, AttnParams& p, cudaStream_t stream,
@@ -1083,6 +1101,8 @@ dard_status launch_attention(const dard_attn_args& a, AttnParams& p, cudaStream_
     e = launch_simt_attention(p, stream);
   } else if (kernel == 4) {
     e = launch_pair_attention(p, stream);
+  } else if (p.persist) {
+    e = launch_persist_attention(p, stream);
   } else {
     e = a.head_dim == 64 ? launch_tc<64>(p, kernel, stream) : launch_tc<128>(p, kernel, stream);
   }

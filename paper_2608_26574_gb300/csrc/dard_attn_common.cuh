@@ -25,7 +25,7 @@ constexpr uint32_t kTmemCols = 512;  // every TMEM column of the SM
 constexpr float kRescaleLog2 = 8.0f;
 constexpr float kRescaleMax = 256.0f;  // 2^kRescaleLog2
 
-// Per-CTA copy of the current block: states, confidences, the shadow maps, and the same
+// Shared copy of the current block: states, confidences, the shadow maps, and the same
 // facts as bit words over block positions (word w = positions 32w .. 32w + 31).
 struct __align__(16) BlockInfo {
   int32_t st[DARD_MAX_BLOCK];
@@ -139,6 +139,60 @@ __device__ void publish_block_info(const AttnParams& p, const SeqDesc& sd, Block
   sm_bar_sync();
   if (lane == 0 && idw != 0xffffffffu) bi.identity = 0;
   sm_bar_sync();
+}
+
+// The same by one whole warp: lane l takes positions l, l + 32, l + 64 and l + 96.
+__device__ void publish_block_info_warp(const AttnParams& p, const SeqDesc& sd, BlockInfo& bi,
+                                        bool report) {
+  const int lane = threadIdx.x & 31;
+  int st[4], pos[4];
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {  // every load first: they are in flight together
+    const int t = 32 * w + lane;
+    st[w] = t < sd.blen ? p.state[sd.blk_off + t] : -1;
+    pos[w] = t < sd.slen ? p.shadow_src[sd.sh_off + t] - sd.b0 : -1;
+    if (t < sd.blen) bi.cf[t] = p.prev_conf[sd.blk_off + t];
+    bi.shrow[t] = INT_MAX;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    const int t = 32 * w + lane;
+    if (st[w] > 2) {
+      if (report && p.status) atomicOr(p.status, DARD_STATUS_BAD_STATE);
+      st[w] = kStateM;
+    }
+    if (t < sd.blen) bi.st[t] = st[w];
+    if (pos[w] >= sd.blen) pos[w] = -1;
+    if (pos[w] >= 0) atomicMin(&bi.shrow[pos[w]], t);
+  }
+  __syncwarp();
+  bool same = true;  // shpos[t] == t for every shadow row of this lane
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    const int t = 32 * w + lane;
+    const bool ok = pos[w] >= 0 && bi.shrow[pos[w]] == t;
+    if (t < sd.slen && !ok && report && p.status) atomicOr(p.status, DARD_STATUS_BAD_SHADOW);
+    bi.shpos[t] = ok ? pos[w] : -1;
+    same = same && (t >= sd.slen || (ok && pos[w] == t));
+  }
+  __syncwarp();
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    const int t = 32 * w + lane;
+    if (bi.shrow[t] == INT_MAX) bi.shrow[t] = -1;
+    const uint32_t mw = __ballot_sync(0xffffffffu, st[w] == kStateM);
+    const uint32_t cw = __ballot_sync(0xffffffffu, st[w] == kStateC);
+    const uint32_t hw = __ballot_sync(0xffffffffu, t < sd.blen && bi.shrow[t] >= 0);
+    if (lane == 0) {
+      bi.m_w[w] = mw;
+      bi.c_w[w] = cw;
+      bi.hs_w[w] = hw;
+    }
+  }
+  const bool identity = __all_sync(0xffffffffu, same) != 0;
+  if (lane == 0) bi.identity = identity;
+  __syncwarp();
 }
 
 __device__ __forceinline__ void load_block_info(const AttnParams& p, const SeqDesc& sd,
@@ -278,7 +332,7 @@ __device__ RowMasks row_masks(const RowInfo& q, const BlockInfo& bi, const SeqDe
 
 constexpr int kTN = 128;  // keys per tile of the tensor-core path
 constexpr int kL2Ahead = 4;  // K/V tiles the CTA-pair kernel prefetches into L2 ahead of its
-                              // TMA loads (the one- and two-tile kernels: none, measured faster)
+                              // TMA loads (the one-CTA kernel: none, measured faster)
 
 static_assert(kTN == kKeyTile, "one key-tile width for the kernels and the planner");
 

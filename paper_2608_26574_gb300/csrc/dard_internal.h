@@ -68,13 +68,27 @@ struct AttnParams {
   int32_t order[DARD_MAX_SEQS];
   int32_t work_prefix[DARD_MAX_SEQS + 1];
   int32_t pair_prefix[DARD_MAX_SEQS + 1];  // the same over pairs of q-tiles
+  // attn_persist's items (plan_items): by_group: each takes two consecutive (q-tile, head)
+  // units of a K/V head's group, laid out K/V head minor; otherwise two consecutive q-tiles
+  // of a head, laid out as pair_prefix.
+  int32_t persist, by_group, total_items;
+  int32_t group;  // hq / hkv
+  uint64_t div_hq, div_hkv, div_group;  // ceil(2^64 / d), 0 for d = 1: exact 31-bit division
+  int32_t item_prefix[DARD_MAX_SEQS + 1];
   SeqDesc seq[DARD_MAX_SEQS];
 };
 
-// The kernel a validated call launches: 1 or 2 (the tensor-core kernel with one or two
-// query tiles per CTA), 3 (the fp32 CUDA-core kernel). Shared by the launcher and by
-// dard_attention_kernel(); reads DARD_ATTN_TC and the current device's SM count.
-int attention_kernel_choice(const dard_attn_args& a, const AttnParams& p);
+// The kernel a validated call launches: 1 or 2 (the tensor-core kernels over single query
+// tiles or over pairs of a head's tiles; p.persist and the items of a persistent launch are
+// then set in p), 3 (the fp32 CUDA-core kernels), 4 (the CTA-pair kernel). Shared by the
+// launcher and by dard_attention_kernel(); reads DARD_ATTN_TC and the current device's SM
+// count.
+int attention_kernel_choice(const dard_attn_args& a, AttnParams& p);
+
+// The persistent tensor-core kernel (dard_attention_persist.cu): its items, CTAs and launch.
+void plan_items(AttnParams& p, bool by_group);
+int persist_ctas(const AttnParams& p);
+cudaError_t launch_persist_attention(const AttnParams& p, cudaStream_t stream);
 
 // The pair kernel (two CTAs per 256-row work item, tcgen05 cta_group::2, head_dim 128,
 // persistent over work items): launch, and the number of clusters a launch uses.
