@@ -77,11 +77,7 @@ static_assert(128 * kTc2SideRegs + 256 * kTc2SoftmaxRegs == kTc2Threads * kTc2La
 static_assert(kTc2Threads * kTc2LaunchRegs <= 65536, "one CTA per SM");
 
 // Named barriers: 0 = __syncthreads, 1 = warps 0-3 (block info), 2 = the 8 softmax warps,
-// then per kernel: attn_tc1 3 + q = the two warps sharing TMEM lane quarter q; attn_tc2
-// 3 + q = the four warps of query tile q.
-__device__ __forceinline__ void tile_bar_sync(int q) {
-  asm volatile("bar.sync %0, 128;" ::"r"(3 + q) : "memory");
-}
+// then in attn_tc1 3 + q = the two warps sharing TMEM lane quarter q.
 
 constexpr int kNS = 2;   // S buffers in TMEM (a ring of 128-column buffers)
 constexpr int kNKV = 3;  // TMA stages for K and for V
@@ -252,54 +248,56 @@ __global__ void __launch_bounds__(kTc1Threads, 1)
   } else if (warp == kWS) {
     // ------------------------------------------------------------ S issuer
     // S_t = Q K_t^T (Q from TMEM, K from shared memory) into ring buffer t % kNS as soon as
-    // K_t has landed and the softmax has read S_{t - kNS} out of that buffer.
-    if (lane == 0) {
-      constexpr uint32_t kIdS = idesc_bf16_f32(kBM, kTN, 0, 0);
-      const uint32_t ak = smem_u32(sK);
-      bool ok = mbar_wait(&ctl.q_full, 0, wlim);
-      for (int t2 = 0; t2 < n_kt && ok && !*abort_flag; ++t2) {
-        const int kb = t2 % kNKV, sb = t2 % kNS;
-        if (t2 >= kNS) ok = mbar_wait(&ctl.s_free[sb], ((t2 - kNS) / kNS) & 1, wlim);
-        ok = ok && mbar_wait(&ctl.k_full[kb], (t2 / kNKV) & 1, wlim);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t kaddr = ak + kb * kKVBytes;
-        const uint32_t dst = ctl.tmem_base + sb * kTN;
+    // K_t has landed and the softmax has read S_{t - kNS} out of that buffer. As in attn_tc2,
+    // the whole warp runs the loop and an elected lane issues.
+    constexpr uint32_t kIdS = idesc_bf16_f32(kBM, kTN, 0, 0);
+    const uint64_t dk = smem_desc_sw128(smem_u32(sK), 16, 1024);
+    bool ok = warp_wait(&ctl.q_full, 0, wlim);
+    for (int t2 = 0; t2 < n_kt && ok; ++t2) {
+      const int kb = t2 % kNKV, sb = t2 % kNS;
+      if (t2 >= kNS) ok = warp_wait(&ctl.s_free[sb], ((t2 - kNS) / kNS) & 1, wlim);
+      ok = ok && warp_wait(&ctl.k_full[kb], (t2 / kNKV) & 1, wlim);
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t db = dk + kb * (kKVBytes >> 4);
+      const uint32_t dst = ctl.tmem_base + sb * kTN;
+      if (elect_one()) {
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-          const uint32_t ko = (ks >> 2) * kKSub + (ks & 3) * 32;
-          mma_ts(dst, tQ + ks * 8, smem_desc_sw128(kaddr + ko, 16, 1024), kIdS, ks > 0);
-        }
+        for (int ks = 0; ks < D / 16; ++ks)
+          mma_ts(dst, tQ + ks * 8, db + (((ks >> 2) * kKSub + (ks & 3) * 32) >> 4), kIdS, ks > 0);
         mma_commit(&ctl.s_full[sb]);
         mma_commit(&ctl.k_empty[kb]);
       }
-      if (!ok) flag_timeout(p, ctl);
-      mma_commit(&ctl.drained);  // completes once every S product this thread issued has
+      __syncwarp();
     }
+    if (!ok && lane == 0) flag_timeout(p, ctl);
+    if (elect_one()) mma_commit(&ctl.drained);  // completes once every S product issued has
+    __syncwarp();
   } else if (warp == kWPV) {
     // ------------------------------------------------------------ PV issuer
     // O += P_j V_j as soon as the softmax has written P_j and V_j has landed.
-    if (lane == 0) {
-      constexpr uint32_t kIdO = idesc_bf16_f32(kBM, D, 0, 1);
-      const uint32_t av = smem_u32(sV);
-      bool ok = true;
-      for (int j = 0; j < n_kt && ok && !*abort_flag; ++j) {
-        const int vb = j % kNKV;
-        ok = mbar_wait(&ctl.p_full, j & 1, wlim) && mbar_wait(&ctl.v_full[vb], (j / kNKV) & 1, wlim);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t vaddr = av + vb * kKVBytes;
+    constexpr uint32_t kIdO = idesc_bf16_f32(kBM, D, 0, 1);
+    const uint64_t dv = smem_desc_sw128(smem_u32(sV), kKSub, 1024);
+    bool ok = true;
+    for (int j = 0; j < n_kt && ok; ++j) {
+      const int vb = j % kNKV;
+      ok = warp_wait(&ctl.p_full, j & 1, wlim) && warp_wait(&ctl.v_full[vb], (j / kNKV) & 1, wlim);
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t db = dv + vb * (kKVBytes >> 4);
+      if (elect_one()) {
 #pragma unroll
         for (int ks = 0; ks < kTN / 16; ++ks)
-          mma_ts(tO, tP + ks * 8, smem_desc_sw128(vaddr + ks * 2048, kKSub, 1024), kIdO,
-                 (j > 0 || ks > 0) ? 1u : 0u);
+          mma_ts(tO, tP + ks * 8, db + ks * (2048 >> 4), kIdO, (j > 0 || ks > 0) ? 1u : 0u);
         mma_commit(&ctl.pv_done);
         mma_commit(&ctl.v_empty[vb]);
         if (j == n_kt - 1) mma_commit(&ctl.o_full);
       }
-      if (!ok) flag_timeout(p, ctl);
-      mma_commit(&ctl.drained);  // completes once every PV product this thread issued has
+      __syncwarp();
     }
+    if (!ok && lane == 0) flag_timeout(p, ctl);
+    if (elect_one()) mma_commit(&ctl.drained);  // completes once every PV product issued has
+    __syncwarp();
   } else {
     // ------------------------------------------------------------ softmax + epilogue
     const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
@@ -564,7 +562,6 @@ struct __align__(16) Tc2Ctl {
   uint32_t tmem_base;
   int32_t abort;
   BlockInfo bi;
-  uint8_t store_row[kQT][kBM];  // epilogue: rows of each tile that are written
 };
 
 template <int D>
@@ -909,43 +906,37 @@ __global__ void __launch_bounds__(kTc2Threads, 1)
       const bool wok = __all_sync(0xffffffffu, ok);
       if (!wok && lane == 0) flag_timeout(p, ctl);
       // O row / row sum -> bf16 into the tile's query buffer (no MMA reads it once o_full
-      // has completed), 16-byte chunks XOR-swizzled by row; then the tile's 128 threads
-      // store whole rows, coalesced.
+      // has completed), 16-byte chunks XOR-swizzled by row; then each warp stores its own 32
+      // rows, coalesced, without waiting for the others.
       constexpr int kChunks = D / 8;  // 16-byte chunks per output row
       uint4* stage = reinterpret_cast<uint4*>(sQ + q * kTileBytes);
+      const uint32_t rows_out = __ballot_sync(0xffffffffu, ri.store && r < rows_seq);
       if (wok) {
         tc_fence_after();
         const float inv_l = 1.0f / l_run;
+        uint32_t rr[D];
 #pragma unroll
-        for (int c = 0; c < D / 32; ++c) {
-          uint32_t rr[32];
-          tmem_ld32(tO + lane_off + 32 * c, rr);
-          tmem_wait_ld();
+        for (int c = 0; c < D / 32; ++c)
+          tmem_ld32(tO + lane_off + 32 * c, *reinterpret_cast<uint32_t(*)[32]>(rr + 32 * c));
+        tmem_wait_ld();
 #pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            uint4 u;
-            u.x = pack_bf16x2(__uint_as_float(rr[8 * v + 0]) * inv_l, __uint_as_float(rr[8 * v + 1]) * inv_l);
-            u.y = pack_bf16x2(__uint_as_float(rr[8 * v + 2]) * inv_l, __uint_as_float(rr[8 * v + 3]) * inv_l);
-            u.z = pack_bf16x2(__uint_as_float(rr[8 * v + 4]) * inv_l, __uint_as_float(rr[8 * v + 5]) * inv_l);
-            u.w = pack_bf16x2(__uint_as_float(rr[8 * v + 6]) * inv_l, __uint_as_float(rr[8 * v + 7]) * inv_l);
-            const int chunk = c * 4 + v;
-            stage[t * kChunks + (chunk ^ (t & (kChunks - 1)))] = u;
-          }
+        for (int c = 0; c < kChunks; ++c) {
+          uint32_t w[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            w[e] = pack_bf16x2(__uint_as_float(rr[8 * c + 2 * e]) * inv_l,
+                               __uint_as_float(rr[8 * c + 2 * e + 1]) * inv_l);
+          stage[t * kChunks + (c ^ (t & (kChunks - 1)))] = make_uint4(w[0], w[1], w[2], w[3]);
         }
-      }
-      ctl.store_row[q][t] = (wok && ri.store && r < rows_seq) ? 1 : 0;
-      tile_bar_sync(q);
-      if (!*abort_flag) {
+        __syncwarp();
         __nv_bfloat16* out = static_cast<__nv_bfloat16*>(p.o);
         const int rbase = row0 + sd.q_start + (qt0 + q) * kBM;
 #pragma unroll 4
-        for (int idx = t; idx < kBM * kChunks; idx += kBM) {
-          const int row = idx / kChunks, chunk = idx % kChunks;
-          if (ctl.store_row[q][row]) {
+        for (int idx = lane; idx < 32 * kChunks; idx += 32) {
+          const int row = quarter * 32 + idx / kChunks, chunk = idx % kChunks;
+          if ((rows_out >> (idx / kChunks)) & 1u) {
             const uint4 u = stage[row * kChunks + (chunk ^ (row & (kChunks - 1)))];
-            uint4* dst = reinterpret_cast<uint4*>(
-                out + (static_cast<size_t>(rbase + row) * p.hq + h) * D);
-            dst[chunk] = u;
+            reinterpret_cast<uint4*>(out + (static_cast<size_t>(rbase + row) * p.hq + h) * D)[chunk] = u;
           }
         }
       }
