@@ -45,7 +45,8 @@
 //   the common tile (217 us).
 // Both keep a per-row running maximum and rescale O in TMEM only when the maximum grows by
 // more than a factor 2^8 (the exponentials stay bounded by 2^8 otherwise).
-// fp32 path: attn_simt (dard_attention_simt.cu), CUDA cores, the same mask logic.
+// fp32 paths: attn_simt (dard_attention_simt.cu) and attn_f32 (dard_attention_f32.cu), CUDA
+// cores, the same mask logic.
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
@@ -1089,7 +1090,12 @@ dard_status launch_attention(const dard_attn_args& a, AttnParams& p, cudaStream_
     }
   }
   if (kernel == 3) {
-    e = launch_simt_attention(p, stream);
+    // Beyond one wave of attn_simt's CTAs its shared-memory loads bound it: attn_f32 holds 8 x
+    // 2 scores per thread instead of one. Up to there attn_simt's four key groups per CTA
+    // finish sooner. Measured, us (attn_simt, attn_f32) by 128-row tiles x heads at head_dim
+    // 128: 24 130 / 142 (700 keys), 64 160 / 92 (400), 72 356 / 199 (1000), 160 390 / 165 (500).
+    e = p.total_work * kSimtCtasPerTile <= sm_count() ? launch_simt_attention(p, stream)
+                                                      : launch_f32_attention(p, stream);
   } else if (kernel == 4) {
     e = launch_pair_attention(p, stream);
   } else if (p.persist) {

@@ -1,7 +1,7 @@
 """GPU parity of the attention kernels of larger launches: the persistent tensor-core kernel
 (more than one work item per SM: odd head groups, lone tiles, sequences down to one row, query
-starts, several sequences per CTA), with RoPE in the call and without; a wait that runs out in
-a persistent launch."""
+starts, several sequences per CTA) and the fp32 kernel for more than one wave of query tiles,
+with RoPE in the call and without; a wait that runs out in a persistent launch."""
 import numpy as np
 import pytest
 import torch
@@ -61,6 +61,23 @@ def test_persistent_items(d, rope, tc, monkeypatch):
         if rope else P.compare_attention(wl, 0, o, sample=24)
     print("persistent", d, rope, tc, plan, mx, mean, n)
     assert mx <= P.att_tol(wl) and mean <= P.ATT_MEAN_ABS
+
+
+@pytest.mark.parametrize("probe", [False, True])
+@pytest.mark.parametrize("rope", [0, 1, 2])
+@pytest.mark.parametrize("d", [64, 128])
+def test_fp32_larger_launch(d, rope, probe):
+    """fp32 throughout, as for the small calls: 2e-4 of the largest value; with Q = 0 every
+    attended key weighs 1/N, and a wrong one would move the output by far more than 0.25 / N."""
+    if probe and rope:
+        pytest.skip("Q = 0 has nothing to rotate")
+    wl = W.custom(_specs(20 + d, not rope), 12, 4, d, dtype="f32", seed=50 + d + rope, probe=probe,
+                  qkv_std=1.0)
+    _, o = _run(wl, ROPE[rope])
+    mx, mean, n = P.compare_attention(wl, 0, o, sample=None if probe else 24, rope=ROPE[rope])
+    print("fp32", d, rope, probe, mx, mean, n)
+    vmax = max(1.0, float(np.abs(wl.v[0]).max()))
+    assert mx <= (0.25 / max(LENGTHS) if probe else 2e-4 * vmax)
 
 
 @pytest.mark.parametrize("tc", ["1", "2"])
