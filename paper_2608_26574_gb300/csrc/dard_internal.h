@@ -143,7 +143,9 @@ struct ScoreParams {
 
 constexpr int kScoreThreads = 256;
 constexpr int kScoreMaxSplit = 16;  // CTAs per row = thread-block cluster size
-constexpr int kScoreCtasPerSm = 12;  // target CTAs per SM when choosing the split
+// Target CTAs per SM when choosing the split. Measured at 12, 8, 6 and 4 (us): 128 rows of
+// 151643 fp32 logits 22.0, 20.4, 21.7, 24.0; 1024 rows of 126464 bf16 logits 72.0 at each.
+constexpr int kScoreCtasPerSm = 8;
 
 // Validates a scoring call and fills its kernel parameters; touches no device memory.
 dard_status prepare_score(const dard_score_args* a, ScoreParams& p);
