@@ -13,8 +13,9 @@ namespace {
 // vectors 16 v + 4 part .. 16 v + 4 part + 3 (v = 0 .. D/16 - 1) of q and of its O
 // accumulator, so that the row's four threads read 64 contiguous bytes of a shared-memory
 // key row per vector (one 16-byte load each, no bank conflict). The sequence's keys pass
-// through shared memory 32 rows at a time (K and V, read as broadcasts; each thread loads
-// its share of the next tile while the current one is computed); key group `grp` takes
+// through shared memory 32 rows at a time (K and V, read as broadcasts; four tiles in
+// flight by cp.async, the first four issued before the block's metadata is read, so that a
+// short sequence waits for memory once); key group `grp` takes
 // keys 8 grp .. 8 grp + 7 of every tile, four at a time: four independent partial dot
 // products, which the row's four threads add up with two shuffles each, then one online
 // softmax step over the four. At the end the four groups' (maximum, sum, accumulator) of a
@@ -25,19 +26,23 @@ constexpr int kSimtParts = 4;     // threads per query row and key group
 constexpr int kSimtGroups = 4;    // key groups
 constexpr int kSimtGroupThreads = kSimtRows * kSimtParts;
 constexpr int kSimtThreads = kSimtGroupThreads * kSimtGroups;
+constexpr int kSimtStages = 4;    // K/V tiles in shared memory
+constexpr int kSimtKeys = 32;     // keys per tile
 constexpr int kSimtSplit = kSimtCtasPerTile;  // CTAs per 128-row query tile
 static_assert(kSimtSplit * kSimtRows == kBM, "the CTAs cover a 128-row query tile");
 
 template <int D>
 __global__ void __launch_bounds__(kSimtThreads) attn_simt(const __grid_constant__ AttnParams p) {
   constexpr int kV = D / 16;                   // float4 vectors per thread
-  constexpr int kKT = 32;                      // keys per shared-memory tile
+  constexpr int kKT = kSimtKeys;               // keys per shared-memory tile
   constexpr int kKG = kKT / kSimtGroups;       // keys of a tile per key group
   static_assert(kKG % 4 == 0, "four keys per step");
   static_assert(kKT >= kSimtRows, "the merge reuses the K and V tile buffers, one row block each");
   __shared__ BlockInfo bi;
-  __shared__ __align__(16) float sK[kKT][D];
-  __shared__ __align__(16) float sV[kKT][D];
+  extern __shared__ __align__(16) float smem[];  // kSimtStages tiles of K, then of V
+  using Tile = float[kKT][D];
+  Tile* const sKs = reinterpret_cast<Tile*>(smem);
+  Tile* const sVs = sKs + kSimtStages;
   __shared__ float s_m[kSimtGroups][kSimtRows], s_l[kSimtGroups][kSimtRows];
   int seq, qt, h;
   decode_work(p, blockIdx.x / kSimtSplit, seq, qt, h);
@@ -45,6 +50,29 @@ __global__ void __launch_bounds__(kSimtThreads) attn_simt(const __grid_constant_
   const SeqDesc sd = p.seq[seq];
   const int rows_seq = sd.n_orig + sd.slen;
   const int g = h / (p.hq / p.hkv);
+  const float* K = static_cast<const float*>(p.k);
+  const float* V = static_cast<const float*>(p.v);
+  // K and V of keys kt0 .. kt0 + 31 into stage st (rows past the sequence as zeros); every
+  // thread commits one group per tile, copies or none
+  auto copy_tile = [&](int kt0, int st) {
+#pragma unroll
+    for (int u = 0; u < kKT * D / 4 / kSimtThreads; ++u) {
+      const int idx = static_cast<int>(threadIdx.x) + u * kSimtThreads;
+      const int kr = kt0 + idx / (D / 4), c4 = idx % (D / 4);
+      if (kt0 >= rows_seq) break;
+      const bool in = kr < rows_seq;
+      const size_t off =
+          (static_cast<size_t>(sd.row_base + (in ? kr : 0)) * p.hkv + g) * D + 4 * c4;
+      cp_async16(&sKs[st][0][0] + 4 * idx, K + off, in ? 16 : 0);
+      cp_async16(&sVs[st][0][0] + 4 * idx, V + off, in ? 16 : 0);
+    }
+    cp_async_commit();
+  };
+  static_assert(kKT * D / 4 % kSimtThreads == 0, "a tile splits evenly over the threads");
+  // the first tiles before anything else: they land while the block is read
+  grid_dep_wait();  // the RoPE key pass launched before this kernel (if any) is complete
+#pragma unroll
+  for (int st = 0; st < kSimtStages; ++st) copy_tile(st * kKT, st);
   if (threadIdx.x < 128)  // warps 0-3
     load_block_info(p, sd, bi, qt == 0 && h == 0 && sub == 0);
   __syncthreads();
@@ -57,8 +85,6 @@ __global__ void __launch_bounds__(kSimtThreads) attn_simt(const __grid_constant_
   if (active) q = row_info(sd, bi, r);
   const bool live = active && q.store;
   const float* Q = static_cast<const float*>(p.q);
-  const float* K = static_cast<const float*>(p.k);
-  const float* V = static_cast<const float*>(p.v);
   float* O = static_cast<float*>(p.o);
   // vector v of this thread: float4 index 4 v + part of the row
   const size_t qoff4 = (static_cast<size_t>(sd.row_base + r) * p.hq + h) * (D / 4) + part;
@@ -103,38 +129,18 @@ __global__ void __launch_bounds__(kSimtThreads) attn_simt(const __grid_constant_
       }
     }
   }
-  grid_dep_wait();  // the RoPE key pass launched before this kernel (if any) is complete
-  // K/V tiles are software-pipelined: each thread holds its share of the next tile in
-  // registers, loaded while the current tile is computed
-  constexpr int kLoads = kKT * D / 4 / kSimtThreads;  // float4 of K (and of V) per thread
-  static_assert(kKT * D / 4 % kSimtThreads == 0, "a tile splits evenly over the threads");
-  float4 nxk[kLoads], nxv[kLoads];
-  auto fetch = [&](int kt0) {
-#pragma unroll
-    for (int u = 0; u < kLoads; ++u) {
-      const int idx = static_cast<int>(threadIdx.x) + u * kSimtThreads;
-      const int kr = kt0 + idx / (D / 4), c4 = idx % (D / 4);
-      nxk[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      nxv[u] = nxk[u];
-      if (kr < rows_seq) {
-        const size_t off = (static_cast<size_t>(sd.row_base + kr) * p.hkv + g) * (D / 4) + c4;
-        nxk[u] = reinterpret_cast<const float4*>(K)[off];
-        nxv[u] = reinterpret_cast<const float4*>(V)[off];
-      }
-    }
-  };
-  fetch(0);
   float m = -INFINITY, l = 0.f;
-  for (int kt0 = 0; kt0 < rows_seq; kt0 += kKT) {
-    __syncthreads();  // the previous tile has been read
-#pragma unroll
-    for (int u = 0; u < kLoads; ++u) {
-      const int idx = static_cast<int>(threadIdx.x) + u * kSimtThreads;
-      reinterpret_cast<float4*>(sK[idx / (D / 4)])[idx % (D / 4)] = nxk[u];
-      reinterpret_cast<float4*>(sV[idx / (D / 4)])[idx % (D / 4)] = nxv[u];
+  for (int kt0 = 0, t0 = 0; kt0 < rows_seq; kt0 += kKT, ++t0) {
+    if (t0 > 0 && kt0 + (kSimtStages - 1) * kKT < rows_seq) {
+      __syncthreads();  // the tile before has been read: its stage takes the tile kSimtStages on
+      copy_tile(kt0 + (kSimtStages - 1) * kKT, (t0 - 1) % kSimtStages);
+    } else if (t0 > 0) {
+      cp_async_commit();
     }
-    __syncthreads();
-    if (kt0 + kKT < rows_seq) fetch(kt0 + kKT);
+    cp_async_wait<kSimtStages - 1>();
+    __syncthreads();  // this tile has landed
+    const auto& sK = sKs[t0 % kSimtStages];
+    const auto& sV = sVs[t0 % kSimtStages];
     if (!live) continue;
     const int k_end = min(kKT, rows_seq - kt0);
     // four keys per step: four independent dot-product chains, one maximum and at most one
@@ -200,6 +206,8 @@ __global__ void __launch_bounds__(kSimtThreads) attn_simt(const __grid_constant_
   // Merge the key groups: groups 2 and 3 hand their state to groups 0 and 1, then group 1
   // to group 0, through the K and V tile buffers (free once every group is past its last
   // tile): group half + k writes into buffer k (sK for k = 0, sV for k = 1).
+  Tile& sK = sKs[0];
+  Tile& sV = sVs[0];
   if (part == 0) {
     s_m[grp][t] = m;
     s_l[grp][t] = l;
@@ -246,12 +254,20 @@ __global__ void __launch_bounds__(kSimtThreads) attn_simt(const __grid_constant_
   }
 }
 
+template <int D>
+cudaError_t launch_simt(const AttnParams& p, cudaStream_t stream) {
+  static std::atomic<uint64_t> attr_done{0};
+  const size_t smem = 2 * kSimtStages * kSimtKeys * D * sizeof(float);
+  const cudaError_t e = ensure_smem_attr(attn_simt<D>, smem, attr_done);
+  if (e != cudaSuccess) return e;
+  const AttnLaunch L(p.total_work * kSimtSplit, kSimtThreads, smem, stream, 1, p.rope != 0);
+  return cudaLaunchKernelEx(&L.cfg, attn_simt<D>, p);
+}
+
 }  // namespace
 
 cudaError_t launch_simt_attention(const AttnParams& p, cudaStream_t stream) {
-  const AttnLaunch L(p.total_work * kSimtSplit, kSimtThreads, 0, stream, 1, p.rope != 0);
-  return p.head_dim == 64 ? cudaLaunchKernelEx(&L.cfg, attn_simt<64>, p)
-                          : cudaLaunchKernelEx(&L.cfg, attn_simt<128>, p);
+  return p.head_dim == 64 ? launch_simt<64>(p, stream) : launch_simt<128>(p, stream);
 }
 
 }  // namespace dard
