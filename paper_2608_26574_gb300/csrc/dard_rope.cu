@@ -6,11 +6,11 @@
 // (griddepcontrol) before its first key load, and rotates its own query tiles as it loads
 // them. Positions and arithmetic: dard_rope.cuh.
 //
-// One thread per (row, group of four frequencies, four heads): the four cos/sin pairs are
-// formed once and applied to the thread's elements of each of its heads. Interleaved
-// pairing: a group is eight consecutive elements; half pairing: four elements of the first
-// half and the four D/2 later. Consecutive threads take consecutive groups of one row and
-// head, so a warp reads and writes whole 16-byte runs.
+// One thread per (row, group of eight frequencies, four heads): the eight cos/sin pairs are
+// formed once, while the thread's loads are in flight, and applied to its elements of each of
+// its heads. Interleaved pairing: a group is 16 consecutive elements; half pairing: eight
+// elements of the first half and the eight D/2 later. All loads and stores are 16 bytes.
+// Bound: memory (each key row read and written once).
 #include <cuda_bf16.h>
 
 #include "dard_ptx.cuh"
@@ -39,10 +39,44 @@ __device__ __forceinline__ void rot(float& a, float& b, float c, float s) {
   b = fmaf(x, s, y * c);
 }
 
+// Eight values of T as 16-byte vectors, to and from floats.
+template <typename T>
+struct Eight {
+  static constexpr int kVecs = 8 * sizeof(T) / 16;
+  uint4 u[kVecs];
+  __device__ void load(const T* p) {
+#pragma unroll
+    for (int k = 0; k < kVecs; ++k) u[k] = reinterpret_cast<const uint4*>(p)[k];
+  }
+  __device__ void store(T* p) const {
+#pragma unroll
+    for (int k = 0; k < kVecs; ++k) reinterpret_cast<uint4*>(p)[k] = u[k];
+  }
+  __device__ void get(float (&x)[8]) const {
+    const uint32_t* w = &u[0].x;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      if constexpr (sizeof(T) == 2) x[e] = (e & 1) ? bf_hi(w[e / 2]) : bf_lo(w[e / 2]);
+      else x[e] = __uint_as_float(w[e]);
+    }
+  }
+  __device__ void set(const float (&x)[8]) {
+    uint32_t* w = &u[0].x;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      if constexpr (sizeof(T) == 2) {
+        if (e & 1) w[e / 2] = bf_pack(x[e - 1], x[e]);
+      } else {
+        w[e] = __float_as_uint(x[e]);
+      }
+    }
+  }
+};
+
 template <typename T, int D>
 __global__ void __launch_bounds__(kRopeThreads) rope_keys(const __grid_constant__ AttnParams p) {
   grid_dep_launch();  // the attention kernel may be scheduled; it waits for this grid's end
-  constexpr int kGroups = D / 8;  // groups of four frequencies per row
+  constexpr int kGroups = D / 16;  // groups of eight frequencies per row
   const int hblocks = (p.hkv + kRopeHeads - 1) / kRopeHeads;
   const long long idx = static_cast<long long>(blockIdx.x) * kRopeThreads + threadIdx.x;
   const long long total = static_cast<long long>(p.total_rows) * hblocks * kGroups;
@@ -51,66 +85,59 @@ __global__ void __launch_bounds__(kRopeThreads) rope_keys(const __grid_constant_
   const long long rest = idx / kGroups;
   const int hb = static_cast<int>(rest % hblocks);
   const int row = static_cast<int>(rest / hblocks);
-  const SeqDesc& sd = p.seq[seq_of_row(p, row)];
-  const int pos = rope_position(p, sd, row - sd.row_base);
   const bool half = p.rope_style == DARD_ROPE_HALF;
-  // element offsets of the group within a head: [e0, e0 + 4) and [e1, e1 + 4)
-  const int e0 = half ? 4 * grp : 8 * grp;
-  const int e1 = half ? D / 2 + 4 * grp : 8 * grp + 4;
+  // element offsets of the group within a head: [e0, e0 + 8) and [e1, e1 + 8)
+  const int e0 = half ? 8 * grp : 16 * grp;
+  const int e1 = half ? D / 2 + 8 * grp : 16 * grp + 8;
   const T* src = static_cast<const T*>(p.k_src);
   T* dst = static_cast<T*>(const_cast<void*>(p.k));
   const int h0 = hb * kRopeHeads;
   // every head's loads first (they are independent), then the rotations and the stores
-  float x[kRopeHeads][8];
+  Eight<T> u0[kRopeHeads], u1[kRopeHeads];
 #pragma unroll
   for (int hh = 0; hh < kRopeHeads; ++hh) {
     if (h0 + hh >= p.hkv) break;
     const size_t base = (static_cast<size_t>(row) * p.hkv + h0 + hh) * D;
-    if constexpr (sizeof(T) == 2) {
-      const uint2 u0 = *reinterpret_cast<const uint2*>(src + base + e0);
-      const uint2 u1 = *reinterpret_cast<const uint2*>(src + base + e1);
-      x[hh][0] = bf_lo(u0.x); x[hh][1] = bf_hi(u0.x); x[hh][2] = bf_lo(u0.y); x[hh][3] = bf_hi(u0.y);
-      x[hh][4] = bf_lo(u1.x); x[hh][5] = bf_hi(u1.x); x[hh][6] = bf_lo(u1.y); x[hh][7] = bf_hi(u1.y);
-    } else {
-      const float4 u0 = *reinterpret_cast<const float4*>(src + base + e0);
-      const float4 u1 = *reinterpret_cast<const float4*>(src + base + e1);
-      x[hh][0] = u0.x; x[hh][1] = u0.y; x[hh][2] = u0.z; x[hh][3] = u0.w;
-      x[hh][4] = u1.x; x[hh][5] = u1.y; x[hh][6] = u1.z; x[hh][7] = u1.w;
-    }
+    u0[hh].load(src + base + e0);
+    u1[hh].load(src + base + e1);
   }
   // the angles while the loads are in flight
-  float c[4], s[4];
+  const SeqDesc& sd = p.seq[seq_of_row(p, row)];
+  const int pos = rope_position(p, sd, row - sd.row_base);
+  float c[8], s[8];
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const int i = 4 * grp + e;  // frequency index
+  for (int e = 0; e < 8; ++e) {
+    const int i = 8 * grp + e;  // frequency index
     rope_cos_sin(pos, p.rope_f[2 * i], p.rope_f[2 * i + 1], c[e], s[e]);
   }
 #pragma unroll
   for (int hh = 0; hh < kRopeHeads; ++hh) {
     if (h0 + hh >= p.hkv) break;
-    float* y = x[hh];
+    float x[8], y[8];
+    u0[hh].get(x);
+    u1[hh].get(y);
     if (half) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) rot(y[e], y[4 + e], c[e], s[e]);
+      for (int e = 0; e < 8; ++e) rot(x[e], y[e], c[e], s[e]);
     } else {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) rot(y[2 * e], y[2 * e + 1], c[e], s[e]);
+      for (int e = 0; e < 4; ++e) {
+        rot(x[2 * e], x[2 * e + 1], c[e], s[e]);
+        rot(y[2 * e], y[2 * e + 1], c[4 + e], s[4 + e]);
+      }
     }
+    u0[hh].set(x);
+    u1[hh].set(y);
     const size_t base = (static_cast<size_t>(row) * p.hkv + h0 + hh) * D;
-    if constexpr (sizeof(T) == 2) {
-      *reinterpret_cast<uint2*>(dst + base + e0) = make_uint2(bf_pack(y[0], y[1]), bf_pack(y[2], y[3]));
-      *reinterpret_cast<uint2*>(dst + base + e1) = make_uint2(bf_pack(y[4], y[5]), bf_pack(y[6], y[7]));
-    } else {
-      *reinterpret_cast<float4*>(dst + base + e0) = make_float4(y[0], y[1], y[2], y[3]);
-      *reinterpret_cast<float4*>(dst + base + e1) = make_float4(y[4], y[5], y[6], y[7]);
-    }
+    u0[hh].store(dst + base + e0);
+    u1[hh].store(dst + base + e1);
   }
 }
 
 template <typename T>
 cudaError_t launch_typed(const AttnParams& p, cudaStream_t stream) {
   const long long hblocks = (p.hkv + kRopeHeads - 1) / kRopeHeads;
-  const long long threads = static_cast<long long>(p.total_rows) * hblocks * (p.head_dim / 8);
+  const long long threads = static_cast<long long>(p.total_rows) * hblocks * (p.head_dim / 16);
   const long long blocks = (threads + kRopeThreads - 1) / kRopeThreads;
   if (blocks < 1) return cudaSuccess;
   if (blocks > 0x7fffffffll) return cudaErrorInvalidValue;
