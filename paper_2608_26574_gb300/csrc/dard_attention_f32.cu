@@ -2,6 +2,8 @@
 // F32; attn_simt takes the small calls). Same mask as the tensor-core kernels (Sec. 3.1 Eq. 2;
 // Sec. 3.2 query blocks 1-6, Eq. 3) and the same RoPE positions (dard_rope.cuh); fp32 FMAs
 // throughout.
+#include <type_traits>
+
 #include "dard_attn_common.cuh"
 
 namespace dard {
@@ -157,8 +159,9 @@ __global__ void __launch_bounds__(kFThreads) attn_f32(const __grid_constant__ At
     for (int i = 0; i < 8; ++i) {
 #pragma unroll
       for (int c = 0; c < kNC; ++c) z[i][c] *= p.scale;
+      uint64_t vis = ~0ull;
       if (masked) {
-        const uint64_t vis = vis64(sd, kt0, sm.rm[8 * i + ty]) >> tx;
+        vis = vis64(sd, kt0, sm.rm[8 * i + ty]) >> tx;
 #pragma unroll
         for (int c = 0; c < kNC; ++c) z[i][c] = ((vis >> (16 * c)) & 1ull) ? z[i][c] : -INFINITY;
       }
@@ -174,7 +177,10 @@ __global__ void __launch_bounds__(kFThreads) attn_f32(const __grid_constant__ At
       float sum = 0.f;
 #pragma unroll
       for (int c = 0; c < kNC; ++c) {
-        const float w = z[i][c] == -INFINITY ? 0.f : expf(z[i][c] - ref);
+        // a key that the row does not see weighs -0, by which PV leaves it out
+        const float w = !((vis >> (16 * c)) & 1ull) ? -0.f
+                        : z[i][c] == -INFINITY      ? 0.f
+                                                    : expf(z[i][c] - ref);
         sum += w;
         sm.p[8 * i + ty][tx + 16 * c] = w;
       }
@@ -189,29 +195,36 @@ __global__ void __launch_bounds__(kFThreads) attn_f32(const __grid_constant__ At
     for (int i = 0; i < 8; ++i)
 #pragma unroll
       for (int c = 0; c < 2 * kC; ++c) part[i][c] = 0;
+    const auto add_pv = [&](auto tile_masked) {
+      constexpr bool kMasked = decltype(tile_masked)::value;
 #pragma unroll 2
-    for (int kk = 0; kk < kFKeys; kk += 4) {
-      float4 pv[8];
+      for (int kk = 0; kk < kFKeys; kk += 4) {
+        float4 pv[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) pv[i] = *reinterpret_cast<const float4*>(&sm.p[8 * i + ty][kk]);
+        for (int i = 0; i < 8; ++i) pv[i] = *reinterpret_cast<const float4*>(&sm.p[8 * i + ty][kk]);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        ulonglong2 vv[kC];
+        for (int u = 0; u < 4; ++u) {
+          ulonglong2 vv[kC];
 #pragma unroll
-        for (int c = 0; c < kC; ++c)
-          vv[c] = *reinterpret_cast<const ulonglong2*>(&sm.v[kk + u][4 * tx + 64 * c]);
+          for (int c = 0; c < kC; ++c)
+            vv[c] = *reinterpret_cast<const ulonglong2*>(&sm.v[kk + u][4 * tx + 64 * c]);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float w = u == 0 ? pv[i].x : u == 1 ? pv[i].y : u == 2 ? pv[i].z : pv[i].w;
-          const uint64_t w2 = f2_pack(w, w);
+          for (int i = 0; i < 8; ++i) {
+            const float w = u == 0 ? pv[i].x : u == 1 ? pv[i].y : u == 2 ? pv[i].z : pv[i].w;
+            // V of a key that the row does not see may hold anything, a NaN too
+            if (kMasked && __float_as_int(w) == INT_MIN) continue;
+            const uint64_t w2 = f2_pack(w, w);
 #pragma unroll
-          for (int c = 0; c < kC; ++c) {
-            part[i][2 * c] = f2_fma(w2, vv[c].x, part[i][2 * c]);
-            part[i][2 * c + 1] = f2_fma(w2, vv[c].y, part[i][2 * c + 1]);
+            for (int c = 0; c < kC; ++c) {
+              part[i][2 * c] = f2_fma(w2, vv[c].x, part[i][2 * c]);
+              part[i][2 * c + 1] = f2_fma(w2, vv[c].y, part[i][2 * c + 1]);
+            }
           }
         }
       }
-    }
+    };
+    if (masked) add_pv(std::true_type{});
+    else add_pv(std::false_type{});
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll

@@ -101,3 +101,27 @@ def test_wait_runs_out_in_a_persistent_launch(monkeypatch, tc):
     assert int(ds.status.item()) == 0
     mx, mean, _ = P.compare_attention(wl, 0, o.float().cpu().numpy(), sample=8)
     assert mx <= P.ATT_MAX_ABS and mean <= P.ATT_MEAN_ABS
+
+
+@pytest.mark.parametrize("heads", [2, 16])
+@pytest.mark.parametrize("d", [64, 128])
+def test_fp32_hidden_rows_may_hold_anything(d, heads):
+    """A block of settled (U) positions: shadow row j is seen by itself only. With NaN in the first
+    16 shadow keys and values, every other row stays what it is."""
+    n, b0, blen = 512, 256, 32
+    g = torch.Generator("cuda").manual_seed(d + heads)
+    q, k, v = (torch.randn(n + blen, heads, d, generator=g, device="cuda") for _ in range(3))
+    call = B.AttentionCall([n], [b0], [blen], [blen],
+                           torch.full((blen,), 2, dtype=torch.uint8, device="cuda"),
+                           torch.full((blen,), 0.9, device="cuda"),
+                           torch.arange(b0, b0 + blen, dtype=torch.int32, device="cuda"))
+    clean, out = torch.zeros_like(q), torch.zeros_like(q)
+    call(q, k, v, clean)
+    k[n:n + 16] = float("nan")
+    v[n:n + 16] = float("nan")
+    call(q, k, v, out)
+    torch.cuda.synchronize()
+    others = torch.ones(n + blen, dtype=torch.bool, device="cuda")
+    others[n:n + 16] = False
+    assert torch.isfinite(clean).all() and torch.equal(out[others], clean[others])
+    assert torch.isnan(out[~others]).all()
