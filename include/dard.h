@@ -164,9 +164,10 @@ typedef enum { DARD_ROPE_INTERLEAVED = 0, DARD_ROPE_HALF = 1 } dard_rope_style;
 /* Rows are total_rows = sum_i (N_i + S_i). q, k, v, o must be 16-byte aligned; with dtype
  * BF16 a tensor-core kernel runs (head_dim 64 or 128), with F32 the CUDA-core kernel.
  * Of the two ways to make work items of 128-row query tiles (1: single tiles of a K/V head's
- * query heads, each against its own key tiles; 2: two consecutive tiles of one head) the library picks the one a cost model of the batch (query tiles, key tiles,
- * SM count) predicts to be faster; the environment variable DARD_ATTN_TC=1 or 2 forces one of
- * them (results agree within rounding).
+ * query heads, each against its own key tiles; 2: two consecutive tiles of one head) the
+ * library picks the one a cost model of the batch (query tiles, key tiles, SM count) predicts
+ * to be faster; the environment variable DARD_ATTN_TC=1 or 2 forces one of them (results
+ * agree within rounding).
  * Errors: DARD_ERR_NULL (also: k_rope NULL with rope_theta > 0), _SHAPE, _VALUE (scale < 0
  * or not finite; rope_theta neither 0 nor a finite value >= 1; rope_style not a
  * dard_rope_style), _UNSUPPORTED, _ALIGN, _CUDA. */
@@ -188,8 +189,9 @@ dard_status dard_attention_kernel(const dard_attn_args* args, int32_t* kernel);
  * go through the same host validation as dard_step_attention and fail with the same codes.
  *   kernel              as dard_attention_kernel (0: no query rows, nothing launched)
  *   ctas                CTAs of the launch (kernels 1 and 2: at most one per SM, persistent
- *                       beyond one wave; the CTA-pair kernel: two per cluster, as many clusters as fit
- *                       on the current device, or SMs / 2 without one)
+ *                       beyond one wave; the CTA-pair kernel: two per cluster, as many
+ *                       clusters as fit on the current device, or SMs / 2 without one; fp32:
+ *                       four per 128-row query tile and head up to one per SM, else two)
  *   tile_pairs          (query tile, key tile) pairs a tensor-core kernel computes: 128 query
  *                       rows of one head against 128 key rows, over every head and sequence
  *   tile_pairs_skipped  pairs it leaves out because no query of the rows a CTA (or CTA pair)

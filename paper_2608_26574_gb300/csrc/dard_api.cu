@@ -284,7 +284,8 @@ dard_status dard_attention_plan(const dard_attn_args* a, dard_attn_plan* plan) {
   if (p.total_work == 0) return DARD_OK;
   plan->kernel = attention_kernel_choice(*a, p);
   if (plan->kernel == 3) {
-    plan->ctas = static_cast<int64_t>(p.total_work) * kSimtCtasPerTile;
+    plan->ctas = static_cast<int64_t>(p.total_work) *
+                 (simt_suits(p) ? kSimtCtasPerTile : kF32CtasPerTile);
     return DARD_OK;
   }
   plan->ctas = plan->kernel == 4 ? 2ll * pair_clusters_for(p)

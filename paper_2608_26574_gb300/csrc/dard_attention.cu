@@ -69,9 +69,9 @@ constexpr int kWProd = 2 * kQT * 2;  // warp 8: TMA producer
 constexpr int kWMma = kWProd + 1;    // warp 9: TMEM allocator and S issuer
 constexpr int kWPv = kWProd + 2;     // warp 10: PV issuer
 // attn_tc2 register split (setmaxnreg): the launch gives 384 threads 168 registers each; the
-// warpgroup of warps 8-11 (producer, issuers, spare) drops to 56 and the two softmax
-// warpgroups rise to 224, so that a thread holds its row's 128 scores at once:
-// 128 x 56 + 256 x 224 = 384 x 168.
+// warpgroup of warps 8-11 (producer, issuers, spare) drops to 40 and the two softmax
+// warpgroups rise to 232, so that a thread holds its row's 128 scores at once:
+// 128 x 40 + 256 x 232 = 384 x 168.
 constexpr uint32_t kTc2LaunchRegs = 168, kTc2SideRegs = 40, kTc2SoftmaxRegs = 232;
 static_assert(128 * kTc2SideRegs + 256 * kTc2SoftmaxRegs == kTc2Threads * kTc2LaunchRegs,
               "the register shares must add up to the launch's registers");
@@ -1068,6 +1068,14 @@ int attention_kernel_choice(const dard_attn_args& a, AttnParams& p) {
   return kernel;
 }
 
+// Beyond one wave of attn_simt's CTAs its shared-memory loads bound it: attn_f32 holds 8 x 2
+// scores per thread instead of one. Up to there attn_simt's four key groups per CTA finish
+// sooner. Measured, us (attn_simt, attn_f32) by 128-row tiles x heads at head_dim 128: 24
+// 130 / 142 (700 keys), 64 160 / 92 (400), 72 356 / 199 (1000), 160 390 / 165 (500).
+bool simt_suits(const AttnParams& p) {
+  return static_cast<int64_t>(p.total_work) * kSimtCtasPerTile <= sm_count();
+}
+
 dard_status launch_attention(const dard_attn_args& a, AttnParams& p, cudaStream_t stream,
                              char* err, size_t err_len) {
   cudaError_t e;
@@ -1090,12 +1098,7 @@ dard_status launch_attention(const dard_attn_args& a, AttnParams& p, cudaStream_
     }
   }
   if (kernel == 3) {
-    // Beyond one wave of attn_simt's CTAs its shared-memory loads bound it: attn_f32 holds 8 x
-    // 2 scores per thread instead of one. Up to there attn_simt's four key groups per CTA
-    // finish sooner. Measured, us (attn_simt, attn_f32) by 128-row tiles x heads at head_dim
-    // 128: 24 130 / 142 (700 keys), 64 160 / 92 (400), 72 356 / 199 (1000), 160 390 / 165 (500).
-    e = p.total_work * kSimtCtasPerTile <= sm_count() ? launch_simt_attention(p, stream)
-                                                      : launch_f32_attention(p, stream);
+    e = simt_suits(p) ? launch_simt_attention(p, stream) : launch_f32_attention(p, stream);
   } else if (kernel == 4) {
     e = launch_pair_attention(p, stream);
   } else if (p.persist) {

@@ -25,7 +25,7 @@ constexpr int kFRows = 64;   // query rows per CTA
 constexpr int kFKeys = 32;   // keys per tile
 constexpr int kNC = kFKeys / 16;  // keys per thread
 constexpr int kFThreads = 128;
-constexpr int kFPerTile = kBM / kFRows;  // CTAs per 128-row query tile
+static_assert(kF32CtasPerTile * kFRows == kBM, "the CTAs cover a 128-row query tile");
 
 template <int D>
 struct __align__(16) F32Smem {
@@ -43,8 +43,8 @@ __global__ void __launch_bounds__(kFThreads) attn_f32(const __grid_constant__ At
   extern __shared__ __align__(16) uint8_t smem_raw[];
   F32Smem<D>& sm = *reinterpret_cast<F32Smem<D>*>(smem_raw);
   int seq, qt, h;
-  decode_work(p, blockIdx.x / kFPerTile, seq, qt, h);
-  const int sub = blockIdx.x % kFPerTile;
+  decode_work(p, blockIdx.x / kF32CtasPerTile, seq, qt, h);
+  const int sub = blockIdx.x % kF32CtasPerTile;
   const SeqDesc sd = p.seq[seq];
   const int rows_seq = sd.n_orig + sd.slen;
   const int r0 = sd.q_start + qt * kBM + sub * kFRows;  // first (sequence-relative) query row
@@ -260,7 +260,7 @@ cudaError_t launch(const AttnParams& p, cudaStream_t stream) {
   static std::atomic<uint64_t> attr_done{0};
   const cudaError_t e = ensure_smem_attr(attn_f32<D>, sizeof(F32Smem<D>), attr_done);
   if (e != cudaSuccess) return e;
-  const AttnLaunch L(p.total_work * kFPerTile, kFThreads, sizeof(F32Smem<D>), stream, 1, p.rope != 0);
+  const AttnLaunch L(p.total_work * kF32CtasPerTile, kFThreads, sizeof(F32Smem<D>), stream, 1, p.rope != 0);
   return cudaLaunchKernelEx(&L.cfg, attn_f32<D>, p);
 }
 

@@ -96,8 +96,10 @@ cudaError_t launch_pair_attention(const AttnParams& p, cudaStream_t stream);
 // The fp32 CUDA-core attention kernel (dard_attention_simt.cu); kSimtCtasPerTile CTAs per
 // 128-row query tile.
 cudaError_t launch_simt_attention(const AttnParams& p, cudaStream_t stream);
-// The same for more query rows (dard_attention_f32.cu).
+// The same for more query rows (dard_attention_f32.cu); kF32CtasPerTile CTAs per tile.
+constexpr int kF32CtasPerTile = 2;
 cudaError_t launch_f32_attention(const AttnParams& p, cudaStream_t stream);
+bool simt_suits(const AttnParams& p);  // which of the two an fp32 call runs
 int pair_clusters_for(const AttnParams& p);
 
 dard_status launch_attention(const dard_attn_args& a, AttnParams& p, cudaStream_t stream,

@@ -234,3 +234,13 @@ def test_attention_plan_validates_like_the_launch(lib):
     assert lib.dard_attention_plan(ctypes.byref(a), ctypes.byref(out)) == 4
     assert lib.dard_attention_plan(ctypes.byref(a), None) == 1
     assert lib.dard_attention_plan(None, ctypes.byref(out)) == 1
+
+
+def test_attention_plan_counts_the_fp32_ctas(lib):
+    """fp32 CTAs per 128-row query tile and head: four up to one per SM (148 assumed without a
+    device, more on one), two beyond (200 rows and no shadow rows: two tiles per head)."""
+    one = dict(dtype=B.DARD_F32, n=np.array([200], np.int32), b0=np.array([100], np.int32),
+               bl=np.array([32], np.int32), sl=np.array([0], np.int32), head_dim=64)
+    assert _plan(lib, hq=4, hkv=4, **one).ctas == 4 * 2 * 4
+    assert _plan(lib, hq=18, hkv=18, **one).ctas == 4 * 2 * 18
+    assert _plan(lib, hq=20, hkv=20, **one).ctas == 2 * 2 * 20
