@@ -132,8 +132,8 @@ struct __align__(16) PersistCtl {
   // before it in turn), so has stored P_q(n + 1), which waits for PV_q(n): the issuer of PV
   // has taken its slot before the slot's next use.
   uint64_t pv_go[kQT][kPvGo];
-  uint64_t pv_done[kQT];  // PV_q(n) completed: P_q(n + 1) may replace P_q(n)
-  uint64_t o_full[kQT];   // the item's last PV_q completed
+  uint64_t pv_done[kQT];  // PV_q(n) completed: P_q(n + 1) may replace P_q(n), and after an item's
+                          // last key tile O_q is final
   uint64_t drained;       // every product both issuers launched has completed (two commits)
   uint32_t tmem_base;
   int32_t abort;
@@ -282,7 +282,6 @@ __global__ void __launch_bounds__(kPersThreads, 1)
       mbar_init(&ctl.p_full[q], 4);
       for (int b = 0; b < kPvGo; ++b) mbar_init(&ctl.pv_go[q][b], 1);
       mbar_init(&ctl.pv_done[q], 1);
-      mbar_init(&ctl.o_full[q], 1);
     }
     for (int b = 0; b < kNK; ++b) {
       if (b > 0) mbar_init(&ctl.k_full[b], 1);
@@ -445,10 +444,9 @@ __global__ void __launch_bounds__(kPersThreads, 1)
     int n0 = 0, n1 = 0;    // PV products per slot
     int go0 = 0, go1 = 0;  // hand-offs taken per slot
     auto issue = [&](int q, int j, int nk, int& n, int& go, uint64_t db) {
-      const bool last = j == nk - 1;
       if (!warp_wait(&ctl.p_full[q], n & 1, wlim)) return false;
       ++n;
-      if (!last) {
+      if (j < nk - 1) {
         if (!warp_wait(&ctl.pv_go[q][go % kPvGo], (go / kPvGo) & 1, wlim)) return false;
         ++go;
       }
@@ -459,7 +457,6 @@ __global__ void __launch_bounds__(kPersThreads, 1)
         for (int ks = 0; ks < kTN / 16; ++ks)
           mma_ts(td, ta + ks * 8, db + ks * (2048 >> 4), kIdO, (j > 0 || ks > 0) ? 1u : 0u);
         mma_commit(&ctl.pv_done[q]);
-        if (last) mma_commit(&ctl.o_full[q]);
       }
       __syncwarp();
       return true;
@@ -586,7 +583,7 @@ __global__ void __launch_bounds__(kPersThreads, 1)
           raise = true;
         }
         // P_q(n) replaces P_q(n - 1), and O_q may be rescaled, once PV_q(n - 1) has completed
-        // (an item's first tile: its o_full has been waited for)
+        // (an item's first tile: waited for at the end of the item before)
         if (j > 0) ok = mbar_wait(&ctl.pv_done[q], (n - 1) & 1, wlim);
         ++n;
         tc_fence_after();
@@ -610,7 +607,7 @@ __global__ void __launch_bounds__(kPersThreads, 1)
         __syncwarp();
         if (lane == 0) mbar_arrive(&ctl.p_full[q]);
       }
-      if (ok) ok = mbar_wait(&ctl.o_full[q], iq & 1, wlim) &&
+      if (ok) ok = mbar_wait(&ctl.pv_done[q], (n - 1) & 1, wlim) &&
                    mbar_wait(&ctl.bi_full[k % kItems], (k / kItems) & 1, wlim);
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       ++iq;
