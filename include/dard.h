@@ -316,6 +316,19 @@ dard_status dard_score_and_transition(const dard_score_args* args, void* stream)
 #define DARD_SCORE_NOALLOC_MAX_ROWS 8192
 dard_status dard_score_and_transition_noalloc(const dard_score_args* args, void* stream);
 
+/* The elementwise work between a layer's projections, one launch each (interface additions: the
+ * paper has no counterpart). Device pointers, contiguous rows, dtype F32 or BF16, any size and
+ * alignment of the type (16-byte accesses where the rows allow them); arithmetic in fp32.
+ *   dard_add_rmsnorm  s = x + add (add NULL: x), rounded to dtype; sum = s (sum NULL: not
+ *                     stored); out = s / sqrt(mean(s^2) + eps) per row. sum and out may each
+ *                     be x or add.
+ *   dard_swiglu       out = a / (1 + exp(-a)) * b over n elements; out may be a or b.
+ * Errors: DARD_ERR_NULL, _SHAPE, _VALUE, _ALIGN, _CUDA. */
+dard_status dard_add_rmsnorm(const void* x, const void* add, void* sum, void* out, int32_t rows,
+                             int32_t width, int32_t dtype, float eps, void* stream);
+dard_status dard_swiglu(const void* a, const void* b, void* out, int64_t n, int32_t dtype,
+                        void* stream);
+
 /* Human-readable name of a status code; never NULL. */
 const char* dard_status_string(dard_status s);
 

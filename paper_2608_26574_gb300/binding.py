@@ -78,6 +78,10 @@ EXPORTS = {
     "dard_score_and_transition": (ctypes.c_int, [ctypes.POINTER(ScoreArgs), ctypes.c_void_p]),
     "dard_score_and_transition_noalloc": (ctypes.c_int, [ctypes.POINTER(ScoreArgs),
                                                          ctypes.c_void_p]),
+    "dard_add_rmsnorm": (ctypes.c_int, [ctypes.c_void_p] * 4 + [ctypes.c_int32] * 3 +
+                         [ctypes.c_float, ctypes.c_void_p]),
+    "dard_swiglu": (ctypes.c_int, [ctypes.c_void_p] * 3 + [ctypes.c_int64, ctypes.c_int32,
+                                                           ctypes.c_void_p]),
     "dard_score_workspace_size": (ctypes.c_size_t, [ctypes.c_int32, ctypes.c_int32, ctypes.c_int32]),
     "dard_status_string": (ctypes.c_char_p, [ctypes.c_int]),
     "dard_last_error": (ctypes.c_char_p, []),
@@ -403,3 +407,30 @@ def dard_score_and_transition_noalloc(logits_x, logits_s, block_len, state_in, t
     (at most ``SCORE_NOALLOC_MAX_ROWS`` block rows; calls that overlap on one device race)."""
     ScoreCall(block_len, state_in, tau_c, tau_u, lam, p0, conf, token, state_out, None,
               w_out=w_out, counts=counts, status=status)(logits_x, logits_s, stream)
+
+
+def _same(t, like, name: str) -> int | None:
+    """Device pointer of an optional contiguous tensor shaped and typed like ``like``."""
+    if t is None:
+        return None
+    if not t.is_cuda or not t.is_contiguous() or t.shape != like.shape or t.dtype != like.dtype \
+            or t.get_device() != like.get_device():
+        raise ValueError(f"{name}: a contiguous device tensor {tuple(like.shape)} of {like.dtype} expected")
+    return t.data_ptr()
+
+
+def add_rmsnorm(x, out, add=None, sum_out=None, eps: float = 1e-6, stream=None):
+    """``out`` = s / sqrt(mean(s^2) + eps) of each row of s = x + add (or x); s to ``sum_out``."""
+    px = _same(x, x, "x")
+    _check(lib().dard_add_rmsnorm(px, _same(add, x, "add"), _same(sum_out, x, "sum_out"),
+                                  _same(out, x, "out"), x.numel() // x.shape[-1], x.shape[-1],
+                                  _dtype_code(x), eps, _stream_handle(stream, x.get_device())),
+           "dard_add_rmsnorm")
+    return out
+
+
+def swiglu(a, b, out, stream=None):
+    """``out`` = silu(a) * b."""
+    _check(lib().dard_swiglu(_same(a, a, "a"), _same(b, a, "b"), _same(out, a, "out"), a.numel(),
+                             _dtype_code(a), _stream_handle(stream, a.get_device())), "dard_swiglu")
+    return out

@@ -77,6 +77,7 @@ class DLLM:
 
     @staticmethod
     def rmsnorm(x):
+        """RMSNorm as tensor operations (any device and type; ``forward`` uses the kernel)."""
         xf = x.float()
         return (xf * torch.rsqrt(xf.pow(2).mean(-1, keepdim=True) + 1e-6)).to(x.dtype)
 
@@ -94,8 +95,13 @@ class DLLM:
                                     batch.shadow_src, status=batch.status,
                                     rope_theta=cfg.rope_base,
                                     rope_style=B.DARD_ROPE_INTERLEAVED)
+        # Norms (with the residual add before them) and gates are one launch each: as tensor
+        # operations they were 30 of the launches of a layer, and launching took most of the
+        # time of a forward pass (two layers of d_model 1024, 2688 rows).
+        delta = None  # what the layer before adds to h
         for L in self.layers:
-            a = self.rmsnorm(h)
+            a = torch.empty_like(h)
+            B.add_rmsnorm(h, a, delta, None if delta is None else h)
             q = (a @ L["wq"]).view(rows, cfg.hq, cfg.head_dim).contiguous()
             k = (a @ L["wk"]).view(rows, cfg.hkv, cfg.head_dim).contiguous()
             v = (a @ L["wv"]).view(rows, cfg.hkv, cfg.head_dim).contiguous()
@@ -104,16 +110,20 @@ class DLLM:
             attention(q, k, v, o, k_rope=k_rope)
             if need_attn_out:
                 attn_outs.append((q, k, v, o))
-            h = h + o.view(rows, cfg.hq * cfg.head_dim) @ L["wo"]
-            m = self.rmsnorm(h)
-            h = h + (torch.nn.functional.silu(m @ L["w1"]) * (m @ L["w3"])) @ L["w2"]
-        h = self.rmsnorm(h)
-        hx = h[batch.x_rows]
-        hs = h[batch.s_rows]
-        lx = (hx @ self.head) * cfg.logit_scale
-        ls = (hs @ self.head) * cfg.logit_scale
-        return (lx.contiguous(), ls.contiguous(), attn_outs) if need_attn_out else \
-            (lx.contiguous(), ls.contiguous())
+            m = B.add_rmsnorm(h, a, o.view(rows, cfg.hq * cfg.head_dim) @ L["wo"], h)
+            g = m @ L["w1"]
+            delta = B.swiglu(g, m @ L["w3"], g) @ L["w2"]
+        if delta is not None:
+            h += delta
+        # only the block's rows reach the head, both copies in one product
+        hx, hs = h[batch.x_rows], h[batch.s_rows]
+        n = hx.shape[0]
+        hb = torch.empty(n + hs.shape[0], cfg.d_model, dtype=h.dtype, device=h.device)
+        B.add_rmsnorm(hx, hb[:n])
+        B.add_rmsnorm(hs, hb[n:])
+        logits = (hb @ self.head).mul_(cfg.logit_scale)
+        lx, ls = logits[:n], logits[n:]
+        return (lx, ls, attn_outs) if need_attn_out else (lx, ls)
 
 
 @dataclass
