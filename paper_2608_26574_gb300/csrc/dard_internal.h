@@ -145,9 +145,10 @@ struct ScoreParams {
 
 constexpr int kScoreThreads = 256;
 constexpr int kScoreMaxSplit = 16;  // CTAs per row = thread-block cluster size
-// Target CTAs per SM when choosing the split. Measured at 12, 8, 6 and 4 (us): 128 rows of
-// 151643 fp32 logits 22.0, 20.4, 21.7, 24.0; 1024 rows of 126464 bf16 logits 72.0 at each.
-constexpr int kScoreCtasPerSm = 8;
+// Target CTAs per SM when choosing the split. Measured at 8, 12, 16 and 24 (us): 512 rows of
+// 151936 bf16 logits 52.8, 47.2, 48.8, 51.2; 256 of 151936 fp32 ones 47.0, 44.0, 45.4, 47.2; 1024
+// of 100000 bf16 ones 61.1, 61.1, 63.4, 67.5.
+constexpr int kScoreCtasPerSm = 12;
 
 // Validates a scoring call and fills its kernel parameters; touches no device memory.
 dard_status prepare_score(const dard_score_args* a, ScoreParams& p);

@@ -128,9 +128,9 @@ __device__ __forceinline__ uint4 load_vec(const char* row, int e0, int c1) {
 // the position of the maximum only the vector that holds it (its first element's index and its
 // data): the element within it is looked up once, at the end (winner_index). Tracking the
 // vector takes one comparison per vector where tracking the element took one per value, and
-// the passes over many rows are bound by their
-// instructions as much as by memory (1024 rows of 126464 bf16 logits, 388 MB: 75.9 -> 72.0 us;
-// one block with every end-of-step output 10.4 -> 9.5 us). Streaming the rounds through shared
+// the passes over many bf16 rows are bound by
+// their instructions as much as by memory (1024 rows of 126464 bf16 logits, 388 MB: 75.9 -> 72.0
+// us; one block with every end-of-step output 10.4 -> 9.5 us). fp32 rows: see fold_round. Streaming the rounds through shared
 // memory by bulk copies instead, up to 192 KB in flight on an SM, measured no faster (71.4 us).
 template <int kRaw>  // 16-byte vectors of logits behind a vector of scored values
 struct Run {
@@ -153,10 +153,9 @@ __device__ __forceinline__ Run<kRaw> run_init() {
   return r;
 }
 
-// Folds the W scored values x (elements e0 .., from the vectors raw) into the summary.
-template <int W, bool kExtra, int kRaw>
-__device__ __forceinline__ void fold_vec(Run<kRaw>& r, const float (&x)[W], int e0,
-                                         const uint4 (&raw)[kRaw]) {
+// Folds the W scored values x into the summary; `note(vm)` records where the new maximum vm is.
+template <int W, bool kExtra, int kRaw, class NoteFn>
+__device__ __forceinline__ void fold_vals(Run<kRaw>& r, const float (&x)[W], NoteFn note) {
   float vm, vm2 = -INFINITY;
   if constexpr (kExtra) {
     // the two largest, pair by pair
@@ -178,9 +177,7 @@ __device__ __forceinline__ void fold_vec(Run<kRaw>& r, const float (&x)[W], int 
     r.s *= f;
     if (kExtra) r.hx *= f;
     r.m = vm;
-    r.e0 = e0;
-#pragma unroll
-    for (int k = 0; k < kRaw; ++k) r.win[k] = raw[k];
+    note(vm);
   }
   const float mL = r.m == -INFINITY ? 0.f : r.m * kLog2e;
   const uint64_t l2 = f2_pack(kLog2e, kLog2e), nm2 = f2_pack(-mL, -mL);
@@ -207,7 +204,7 @@ __device__ __forceinline__ void fold_vec(Run<kRaw>& r, const float (&x)[W], int 
 // values as the fold did).
 template <int W, int kRaw, class ValsFn>
 __device__ __forceinline__ int winner_index(const Run<kRaw>& r, ValsFn vals) {
-  if (r.e0 == INT_MAX) return INT_MAX;
+  if (W == 4 || r.e0 == INT_MAX) return r.e0;  // fp32: the element itself
   float x[W];
   vals(r.win, x);
   int idx = INT_MAX;
@@ -349,19 +346,49 @@ template <class T, int VPT, bool kExtra, int kRaw, class ValsFn>
 __device__ __forceinline__ void fold_round(Run<kRaw>& r, int base, int limit,
                                            const uint4 (&raw)[kRaw][VPT], ValsFn vals) {
   const bool whole = base + kScoreThreads * VPT * T::W <= limit;
-#pragma unroll
-  for (int v = 0; v < VPT; ++v) {
-    const int e0 = base + (v * kScoreThreads + static_cast<int>(threadIdx.x)) * T::W;
-    uint4 one[kRaw];
+  // element index of value e of the thread's vector v
+  auto at = [&](int v, int e) {
+    return base + (v * kScoreThreads + static_cast<int>(threadIdx.x)) * T::W + e;
+  };
+  auto values = [&](int v, uint4 (&one)[kRaw], float (&x)[T::W]) {
 #pragma unroll
     for (int k = 0; k < kRaw; ++k) one[k] = raw[k][v];
-    float x[T::W];
     vals(one, x);
     if (!whole) {
 #pragma unroll
-      for (int e = 0; e < T::W; ++e) x[e] = e0 + e < limit ? x[e] : -INFINITY;
+      for (int e = 0; e < T::W; ++e) x[e] = at(v, e) < limit ? x[e] : -INFINITY;
     }
-    fold_vec<T::W, kExtra>(r, x, e0, one);
+  };
+  if constexpr (T::W == 4) {
+    // fp32: the round's values at once. With half the values per byte the instructions matter
+    // less, and the registers that a winning vector takes more: the element is looked up
+    // whenever the maximum grows (64 rows of 151936 with every end-of-step output: 18.3 us by
+    // vector, 17.1 so; 512 rows of 151936: 80.7 and 79.7).
+    float x[VPT * 4];
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+      uint4 one[kRaw];
+      float y[4];
+      values(v, one, y);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[4 * v + e] = y[e];
+    }
+    fold_vals<VPT * 4, kExtra>(r, x, [&](float vm) {
+#pragma unroll
+      for (int e = VPT * 4 - 1; e >= 0; --e) r.e0 = x[e] == vm ? at(e / 4, e % 4) : r.e0;
+    });
+  } else {
+#pragma unroll
+    for (int v = 0; v < VPT; ++v) {
+      uint4 one[kRaw];
+      float x[T::W];
+      values(v, one, x);
+      fold_vals<T::W, kExtra>(r, x, [&](float) {
+        r.e0 = at(v, 0);
+#pragma unroll
+        for (int k = 0; k < kRaw; ++k) r.win[k] = one[k];
+      });
+    }
   }
 }
 
@@ -476,7 +503,7 @@ __device__ __forceinline__ void add_count(const ScoreParams& p, int seq, int sta
 
 // kExtra: the call asks for p_cur, next-step tokens or an in-place state update.
 template <class T, int VPT, bool kExtra>
-__global__ void __launch_bounds__(kScoreThreads) score_pass1(const __grid_constant__ ScoreParams p) {
+__global__ void __launch_bounds__(kScoreThreads, T::W == 4 ? 6 : 5) score_pass1(const __grid_constant__ ScoreParams p) {
   // Launched with programmatic dependent launch after whatever kernel precedes the call
   // (the LM head in a model, the attention kernel in the benchmark): this CTA may already be
   // resident, but it touches no memory before that kernel has completed. Only then may
@@ -522,7 +549,7 @@ __global__ void __launch_bounds__(kScoreThreads) score_pass1(const __grid_consta
 }
 
 template <class T, int VPT, bool kExtra>
-__global__ void __launch_bounds__(kScoreThreads, kExtra ? 3 : 4) score_pass2(const __grid_constant__ ScoreParams p) {
+__global__ void __launch_bounds__(kScoreThreads, 4) score_pass2(const __grid_constant__ ScoreParams p) {
   using A = std::conditional_t<kExtra, AccX, Acc>;
   __shared__ A s_acc[kWarps];
   __shared__ float4 s_slots[2 * kScoreMaxSplit];
@@ -994,6 +1021,13 @@ dard_status launch_score(const dard_score_args& a, ScoreParams& p, cudaStream_t 
   const int W = bf16 ? 8 : 4;
   const int per_round = kScoreThreads * 4 * W;
   set_split(p, per_round, split_cap(p.rows));
+  // CTAs of one round only while the launch's fit at once (four to five per SM, about half of the
+  // rows being each pass's): a second wave of them costs its merges again. Two rounds, measured
+  // against one: 128 rows of 100000 bf16 logits 16.5 -> 13.4 us, 256 of 50000 16.6 -> 14.7, 128 of
+  // 50000 fp32 14.4 -> 11.5; with room for all (128 of 50000 bf16) one round stays.
+  if (p.chunk == per_round && p.nsplit > 1 &&
+      static_cast<long long>(p.rows) * p.nsplit > 8ll * sm_count())
+    set_split(p, per_round, (p.nsplit + 1) / 2);
 
   char* ws = static_cast<char*>(a.workspace);
   const size_t cbytes = score_counter_bytes(p.num_seqs);
