@@ -263,7 +263,17 @@ def per_config(dev, hbm, bf16):
     from paper_2608_26574_gb300 import binding as Bd
     from paper_2608_26574_gb300 import workloads as W
     from paper_2608_26574_gb300.device import DeviceStep
-    kernels = {1: "attn_tc1", 2: "attn_tc2", 3: "attn_simt", 4: "attn_pair"}
+
+    def kernel_name(plan, wl):
+        """Kernels 1 and 2 launch a CTA per query tile or pair of a head's tiles, or fewer,
+        persistent ones; fp32 four CTAs per tile (attn_simt) or two."""
+        tiles = [(s.rows - s.query_start + 127) // 128 for s in wl.seqs]
+        if plan["kernel"] == 3:
+            return "attn_simt" if plan["ctas"] == 4 * wl.hq * sum(tiles) else "attn_f32"
+        if plan["kernel"] == 4:
+            return "attn_pair"
+        units = wl.hq * sum(-(-t // plan["kernel"]) for t in tiles)
+        return "attn_persist" if plan["ctas"] < units else "attn_tc%d" % plan["kernel"]
     out = {}
     for name in ("tiny", "8b", "gqa", "ragged", "mm"):
         entry = {}
@@ -280,7 +290,7 @@ def per_config(dev, hbm, bf16):
             flops = W.attention_flops(wl)
             tf = flops / (us * 1e-6) / 1e12
             rec = {"us": us, "tflops": tf, "frac_bf16": tf / bf16 if wl.dtype == "bf16" else None,
-                   "kernel": kernels.get(plan["kernel"], str(plan["kernel"])),
+                   "kernel": kernel_name(plan, wl),
                    "gflop": flops / 1e9, "tile_pairs": plan["tile_pairs"],
                    "tile_pairs_skipped": plan["tile_pairs_skipped"], "input_sets": ns}
             entry["attention_prefix" if prefix else "attention"] = rec
