@@ -548,8 +548,10 @@ __global__ void __launch_bounds__(kScoreThreads, T::W == 4 ? 6 : 5) score_pass1(
   }
 }
 
-template <class T, int VPT, bool kExtra>
-__global__ void __launch_bounds__(kScoreThreads, 4) score_pass2(const __grid_constant__ ScoreParams p) {
+// kCtas per SM: the bf16 variant with end-of-step outputs wants 80 registers (three CTAs), which
+// pays where few CTAs run (launch_pair).
+template <class T, int VPT, bool kExtra, int kCtas>
+__global__ void __launch_bounds__(kScoreThreads, kCtas) score_pass2(const __grid_constant__ ScoreParams p) {
   using A = std::conditional_t<kExtra, AccX, Acc>;
   __shared__ A s_acc[kWarps];
   __shared__ float4 s_slots[2 * kScoreMaxSplit];
@@ -907,11 +909,11 @@ cudaError_t launch_fused(const ScoreParams& p, cudaStream_t stream) {
   return cudaLaunchKernelEx(&cfg, score_fused<T, VPT, kExtra>, p);
 }
 
-template <class T, int VPT, bool kExtra>
+template <class T, int VPT, bool kExtra, int kCtas>
 cudaError_t launch_pair(const ScoreParams& p, cudaStream_t stream) {
   static std::atomic<uint64_t> done1{0}, done2{0};
   cudaError_t e = allow_wide_clusters(score_pass1<T, VPT, kExtra>, done1);
-  if (e == cudaSuccess) e = allow_wide_clusters(score_pass2<T, VPT, kExtra>, done2);
+  if (e == cudaSuccess) e = allow_wide_clusters(score_pass2<T, VPT, kExtra, kCtas>, done2);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.nsplit, p.rows);
@@ -930,7 +932,7 @@ cudaError_t launch_pair(const ScoreParams& p, cudaStream_t stream) {
   e = cudaLaunchKernelEx(&cfg, score_pass1<T, VPT, kExtra>, p);
   if (e != cudaSuccess) return e;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, score_pass2<T, VPT, kExtra>, p);
+  return cudaLaunchKernelEx(&cfg, score_pass2<T, VPT, kExtra, kCtas>, p);
 }
 
 }  // namespace
@@ -1010,7 +1012,14 @@ cudaError_t launch_rows(ScoreParams& p, cudaStream_t stream, int per_round) {
     }
     p = keep;
   }
-  return launch_pair<T, 4, kExtra>(p, stream);
+  // Three CTAs of pass 2 per SM with 80 registers each, or four with 64 and a few spills, by the
+  // CTAs of both passes (about half are pass 2's). Measured (us, bf16 with every output, three
+  // and four): 32 rows of 126464 logits 9.9 and 10.6, 64 of 151936 15.0 and 16.3 (640 CTAs); 64 of
+  // 100000 14.1 and 12.0 (832 CTAs), 1024 of 100000 80.6 and 76.1.
+  if constexpr (kExtra && T::W == 8)
+    if (static_cast<long long>(p.rows) * p.nsplit <= 5ll * sm_count())
+      return launch_pair<T, 4, kExtra, 3>(p, stream);
+  return launch_pair<T, 4, kExtra, 4>(p, stream);
 }
 
 }  // namespace

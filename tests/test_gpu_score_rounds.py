@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+from paper_2608_26574_gb300 import binding as B
 from paper_2608_26574_gb300 import workloads as W
 from paper_2608_26574_gb300.device import DeviceStep
 
@@ -65,3 +66,25 @@ def test_many_rows_ties_and_nonfinite():
     ds, outs = _score(wl, (vocab + 7) // 8 * 8)
     _check(wl, outs)
     assert int(ds.status.item()) & 0x4
+
+
+@pytest.mark.parametrize("block", [58, 59, 93, 94])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_rows_around_the_launch_rules(dtype, block):
+    """13 CTAs of one round per row: either side of 5 CTAs per SM on 152 SMs (the bf16 variant
+    with end-of-step outputs changes) and of 8 (two rounds per CTA from there on)."""
+    specs = [dict(n_orig=140, block_start=10, block_len=block, fractions=(0.4, 0.3, 0.3))]
+    wl = W.custom(specs, 1, 1, 64, dtype=dtype, vocab=13 * ROUND[dtype], seed=block, logit_std=2.0)
+    ds, outs = _score(wl)
+    _check(wl, outs)
+    ent, mar, key = (torch.zeros(block, device="cuda") for _ in range(3))
+    B.dard_score_and_transition(ds.lx, ds.ls, ds.block_len, ds.state, wl.tau_c, wl.tau_u, wl.lam,
+                                wl.p0, ds.conf, ds.token, ds.state_out, ds.workspace,
+                                w_out=ds.w_out, counts=ds.counts, status=ds.status, entropy=ent,
+                                margin=mar, order_key=key, order_mode=B.ORDER_ENTROPY)
+    torch.cuda.synchronize()
+    out = [t.cpu().numpy() for t in (ds.conf, ds.token, ds.state_out, ds.w_out, ds.counts)]
+    P.compare_scores(wl, *out[:3], w_out=out[3], counts=out[4], entropy=ent.cpu().numpy(),
+                     margin=mar.cpu().numpy(), order_key=key.cpu().numpy(),
+                     order_mode=B.ORDER_ENTROPY)
+    assert int(ds.status.item()) == 0
