@@ -4,9 +4,10 @@
 // As separate tensor operations a norm is seven launches and a gate two, each a pass over the
 // activations: a forward pass of small layers spent its time launching them (two layers of
 // d_model 1024 over 2688 rows: about 70 launches, 1246 us). Here a row's residual sum, its mean
-// square and the normalised row are one launch, and so is the gate (759 us for the whole pass). Arithmetic in fp32; the residual
-// sum is rounded to the storage type before it is squared, as the stored sum is what later
-// layers see. Bound: memory (each operand once; the activations of such layers stay in L2).
+// square and the normalised row are one launch, and so is the gate (759 us for the whole
+// pass). Arithmetic in fp32; the residual sum is rounded to the storage type before it is
+// squared, as the stored sum is what later layers see. Bound: memory (each operand once; the
+// activations of such layers stay in L2).
 #include <cuda_bf16.h>
 
 #include <algorithm>
