@@ -52,9 +52,8 @@ __global__ void __launch_bounds__(kSimtThreads) attn_simt(const __grid_constant_
   const int g = h / (p.hq / p.hkv);
   const float* K = static_cast<const float*>(p.k);
   const float* V = static_cast<const float*>(p.v);
-  // K and V of keys kt0 .. kt0 + 31 into stage st (rows past the sequence as zeros); every
-  // thread commits one group per tile, copies or none
-  auto copy_tile = [&](int kt0, int st) {
+  // the rows of keys kt0 .. kt0 + 31 into a stage (rows past the sequence as zeros)
+  auto copy_rows = [&](Tile& dst, const float* src, int kt0) {
 #pragma unroll
     for (int u = 0; u < kKT * D / 4 / kSimtThreads; ++u) {
       const int idx = static_cast<int>(threadIdx.x) + u * kSimtThreads;
@@ -63,16 +62,25 @@ __global__ void __launch_bounds__(kSimtThreads) attn_simt(const __grid_constant_
       const bool in = kr < rows_seq;
       const size_t off =
           (static_cast<size_t>(sd.row_base + (in ? kr : 0)) * p.hkv + g) * D + 4 * c4;
-      cp_async16(&sKs[st][0][0] + 4 * idx, K + off, in ? 16 : 0);
-      cp_async16(&sVs[st][0][0] + 4 * idx, V + off, in ? 16 : 0);
+      cp_async16(&dst[0][0] + 4 * idx, src + off, in ? 16 : 0);
     }
+  };
+  // K and V of a tile into stage st; every thread commits one group per tile, copies or none
+  auto copy_tile = [&](int kt0, int st) {
+    copy_rows(sKs[st], K, kt0);
+    copy_rows(sVs[st], V, kt0);
     cp_async_commit();
   };
   static_assert(kKT * D / 4 % kSimtThreads == 0, "a tile splits evenly over the threads");
-  // the first tiles before anything else: they land while the block is read
-  grid_dep_wait();  // the RoPE key pass launched before this kernel (if any) is complete
+  // The first tiles before anything else: they land while the block is read. With RoPE the keys
+  // come from the pass launched before this kernel, which is waited for only once the block has
+  // been read and the query row rotated (one call of 96 rows and four heads with head_dim 64, us:
+  // waited for first 20.8, so 18.4); V does not depend on it.
 #pragma unroll
-  for (int st = 0; st < kSimtStages; ++st) copy_tile(st * kKT, st);
+  for (int st = 0; st < kSimtStages; ++st) {
+    if (p.rope) copy_rows(sVs[st], V, st * kKT);
+    else copy_tile(st * kKT, st);
+  }
   if (threadIdx.x < 128)  // warps 0-3
     load_block_info(p, sd, bi, qt == 0 && h == 0 && sub == 0);
   __syncthreads();
@@ -127,6 +135,14 @@ __global__ void __launch_bounds__(kSimtThreads) attn_simt(const __grid_constant_
         rot(a.z, b.z, c[2], s[2]);
         rot(a.w, b.w, c[3], s[3]);
       }
+    }
+  }
+  if (p.rope) {
+    grid_dep_wait();  // the key pass is complete
+#pragma unroll
+    for (int st = 0; st < kSimtStages; ++st) {
+      copy_rows(sKs[st], K, st * kKT);
+      cp_async_commit();  // the first group: every V tile so far, and K(0)
     }
   }
   float m = -INFINITY, l = 0.f;
