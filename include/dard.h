@@ -191,7 +191,9 @@ dard_status dard_attention_kernel(const dard_attn_args* args, int32_t* kernel);
  *   ctas                CTAs of the launch (kernels 1 and 2: at most one per SM, persistent
  *                       beyond one wave; the CTA-pair kernel: two per cluster, as many
  *                       clusters as fit on the current device, or SMs / 2 without one; fp32:
- *                       four per 128-row query tile and head up to one per SM, else two)
+ *                       four per 128-row query tile and head while those that hold query rows
+ *                       are at most one per SM (without a device: while all are at most 148),
+ *                       else two)
  *   tile_pairs          (query tile, key tile) pairs a tensor-core kernel computes: 128 query
  *                       rows of one head against 128 key rows, over every head and sequence
  *   tile_pairs_skipped  pairs it leaves out because no query of the rows a CTA (or CTA pair)

@@ -1070,10 +1070,21 @@ int attention_kernel_choice(const dard_attn_args& a, AttnParams& p) {
 
 // Beyond one wave of attn_simt's CTAs its shared-memory loads bound it: attn_f32 holds 8 x 2
 // scores per thread instead of one. Up to there attn_simt's four key groups per CTA finish
-// sooner. Measured, us (attn_simt, attn_f32) by 128-row tiles x heads at head_dim 128: 24
-// 130 / 142 (700 keys), 64 160 / 92 (400), 72 356 / 199 (1000), 160 390 / 165 (500).
+// sooner. What counts is the CTAs that hold query rows (the last tile of a sequence has fewer of
+// 32 rows than four, and the others end at once). Measured on 152 SMs, us (attn_simt, attn_f32 at
+// head_dim 64; at 128): 140 such CTAs, 200 keys 29, 39; 41, 55; 144, 564 keys 61, 84; 96, 119;
+// 152, 1216 keys 121, 160; 195, 231; 96 (of 192), 1064 keys 109, 147; 174, 213; beyond a wave: 156,
+// 1248 keys 273, 164; 418, 237; 154, 324 keys 72, 55; 97, 78. A host without a device plans by the
+// whole grid against 148 SMs.
 bool simt_suits(const AttnParams& p) {
-  return static_cast<int64_t>(p.total_work) * kSimtCtasPerTile <= sm_count();
+  if (device_sms() == 0) return static_cast<int64_t>(p.total_work) * kSimtCtasPerTile <= sm_count();
+  int64_t ctas = 0;
+  for (int s = 0; s < p.num_seqs; ++s) {
+    const SeqDesc& sd = p.seq[s];
+    const int rows = sd.n_orig + sd.slen - sd.q_start;
+    ctas += static_cast<int64_t>((rows + kSimtRows - 1) / kSimtRows) * p.hq;
+  }
+  return ctas <= sm_count();
 }
 
 dard_status launch_attention(const dard_attn_args& a, AttnParams& p, cudaStream_t stream,

@@ -21,7 +21,6 @@ namespace {
 // softmax step over the four. At the end the four groups' (maximum, sum, accumulator) of a
 // row are merged through shared memory. Masking as on the tensor-core path, by
 // key_visible().
-constexpr int kSimtRows = 32;     // query rows per CTA
 constexpr int kSimtParts = 4;     // threads per query row and key group
 constexpr int kSimtGroups = 4;    // key groups
 constexpr int kSimtGroupThreads = kSimtRows * kSimtParts;
@@ -49,6 +48,8 @@ __global__ void __launch_bounds__(kSimtThreads) attn_simt(const __grid_constant_
   const int sub = blockIdx.x % kSimtSplit;
   const SeqDesc sd = p.seq[seq];
   const int rows_seq = sd.n_orig + sd.slen;
+  const int r0 = sd.q_start + qt * kBM + sub * kSimtRows;  // first (sequence-relative) query row
+  if (r0 >= rows_seq) return;
   const int g = h / (p.hq / p.hkv);
   const float* K = static_cast<const float*>(p.k);
   const float* V = static_cast<const float*>(p.v);
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(kSimtThreads) attn_simt(const __grid_constant_
   const int grp = threadIdx.x / kSimtGroupThreads, local = threadIdx.x % kSimtGroupThreads;
   const int t = local / kSimtParts, part = local % kSimtParts;
   const unsigned quad = 0xfu << ((threadIdx.x & 31) & ~3);  // the row's four threads
-  const int r = sd.q_start + qt * kBM + sub * kSimtRows + t;  // sequence-relative query row
+  const int r = r0 + t;  // sequence-relative query row
   const bool active = r < rows_seq;
   RowInfo q{0, kStateU, 0.f, -1, 0};
   if (active) q = row_info(sd, bi, r);

@@ -465,17 +465,23 @@ struct AttnLaunch {
   AttnLaunch& operator=(const AttnLaunch&) = delete;
 };
 
-int sm_count() {
+// SMs of the current device, 0 without one (looked up once per device).
+int device_sms() {
   static std::atomic<int> cache[64];
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   int n = cache[dev].load(std::memory_order_relaxed);
   if (n <= 0) {
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
-      n = 148;
+      return 0;
     cache[dev].store(n, std::memory_order_relaxed);
   }
   return n;
+}
+
+int sm_count() {  // for plans made without a device, 148
+  const int n = device_sms();
+  return n > 0 ? n : 148;
 }
 
 }  // namespace

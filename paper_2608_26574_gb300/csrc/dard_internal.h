@@ -26,7 +26,8 @@ struct SeqDesc {
 
 // Keys per tile of the tensor-core attention kernels.
 constexpr int kKeyTile = 128;
-// CTAs of the fp32 CUDA-core kernel per 128-row query tile (32 rows each).
+// Query rows per CTA of the fp32 CUDA-core kernel, and its CTAs per 128-row query tile.
+constexpr int kSimtRows = 32;
 constexpr int kSimtCtasPerTile = 4;
 
 // Key tiles that query rows [r0, r1) of a sequence need. Original queries of positions after
