@@ -668,11 +668,12 @@ __global__ void __launch_bounds__(kPersThreads, 1)
       const int b = k % kItems;
       ok = k < kItems || warp_wait(&ctl.item_empty[b], (k / kItems - 1) & 1, wlim);
       if (!ok) break;
-      const TcItem it = k == 0 ? first : tc_item(p, k);
-      if (lane == 0) {
-        ctl.item[b] = it;
-        mbar_arrive(&ctl.item_full[b]);
+      TcItem it = first;
+      if (k > 0) {
+        it = tc_item(p, k);
+        if (lane == 0) ctl.item[b] = it;  // (the first is there: its users do not wait)
       }
+      if (lane == 0) mbar_arrive(&ctl.item_full[b]);
       if (it.nq == 0) break;
       publish_block_info_warp(p, it.sd, ctl.bi[b], it.first);
       if (lane == 0) mbar_arrive(&ctl.bi_full[b]);
