@@ -153,6 +153,11 @@ __device__ __forceinline__ Run<kRaw> run_init() {
   return r;
 }
 
+// The reference of a summary with maximum m, in powers of 2. Without a value (m = -inf), and where
+// the product overflows (logits masked by their type's lowest value), it stays finite: such terms
+// then count 0 against any other maximum, not infinity.
+__device__ __forceinline__ float reference(float m) { return fmaxf(m * kLog2e, -FLT_MAX); }
+
 // Folds the W scored values x into the summary; `note(vm)` records where the new maximum vm is.
 template <int W, bool kExtra, int kRaw, class NoteFn>
 __device__ __forceinline__ void fold_vals(Run<kRaw>& r, const float (&x)[W], NoteFn note) {
@@ -179,7 +184,7 @@ __device__ __forceinline__ void fold_vals(Run<kRaw>& r, const float (&x)[W], Not
     r.m = vm;
     note(vm);
   }
-  const float mL = r.m == -INFINITY ? 0.f : r.m * kLog2e;
+  const float mL = reference(r.m);
   const uint64_t l2 = f2_pack(kLog2e, kLog2e), nm2 = f2_pack(-mL, -mL);
   uint64_t s2 = 0, h2 = 0;  // bit pattern 0 = +0.0f
 #pragma unroll
