@@ -824,7 +824,7 @@ __global__ void __launch_bounds__(kTc2Threads, 1)
     const RowInfo ri = row_info(sd, ctl.bi, r);
     const RowMasks rm = row_masks(ri, ctl.bi, sd);
     const float sl = p.scale_log2;
-    float m_run = -INFINITY, l_run = 0.f;
+    float ref = -INFINITY, l_run = 0.f;
     bool ok = active;
     // the key tiles that need the mask (tile_needs_mask): those of the block, [jb0, jb1), and
     // those from jm on
@@ -851,29 +851,28 @@ __global__ void __launch_bounds__(kTc2Threads, 1)
       // P_q(j) replaces P_q(j - 1), and O_q may be rescaled, once PV_q(j - 1) has completed:
       // asked early, it seldom has to be waited for below
       const bool pv_ok = j == 0 || mbar_try_wait(&ctl.pv_done[q], (j - 1) & 1);
-      // The reference maximum: that of the first tile with a finite score.
-      if (__any_sync(0xffffffffu, m_run == -INFINITY)) {
-        const float mt = tile_row_max(sv);
-        if (m_run == -INFINITY) m_run = mt;
+      // The reference (in powers of two): the maximum of the first tile with a finite score.
+      if (__any_sync(0xffffffffu, ref == -INFINITY)) {
+        const float top = tile_row_max(sv) * sl;
+        if (ref == -INFINITY) ref = top;
       }
-      // The tile's weights against the reference so far. Their sum stays below
-      // 2^kRescaleLog2 unless the tile's maximum exceeds the reference by more than that in
-      // probability; only then is the maximum formed, the reference raised to it, the
-      // weights computed again and O rescaled.
+      // The tile's weights against the reference so far. Only where their sum comes out at
+      // kRescaleMax or more is the maximum formed and the reference raised beyond it, the
+      // weights are computed again and O is rescaled.
       const uint64_t sl2 = f2_pack(sl, sl);
-      const float mL = m_run == -INFINITY ? 0.f : m_run * sl;
+      const float mL = ref == -INFINITY ? 0.f : ref;
       uint64_t nmL2 = f2_pack(-mL, -mL);
       uint32_t pk[64];
       float ls = tile_row_exp(sv, sl2, nmL2, pk);
       float alpha = 1.f;
       bool rescale = false;
       if (__any_sync(0xffffffffu, !(ls < kRescaleMax))) {
-        const float mt = tile_row_max(sv);
-        if ((mt - m_run) * sl > kRescaleLog2) {
+        const float top = tile_row_max(sv) * sl;
+        if (!(ls < kRescaleMax) && top > ref) {  // (no other row matters)
           rescale = true;
-          alpha = ex2_approx((m_run - mt) * sl);
-          m_run = mt;
-          nmL2 = f2_pack(-m_run * sl, -m_run * sl);
+          alpha = ex2_approx(ref - (top + kRaiseRoom));
+          ref = top + kRaiseRoom;
+          nmL2 = f2_pack(-ref, -ref);
         }
         ls = tile_row_exp(sv, sl2, nmL2, pk);
       }

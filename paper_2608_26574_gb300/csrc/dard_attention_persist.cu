@@ -519,7 +519,7 @@ __global__ void __launch_bounds__(kPersThreads, 1)
         if (lane == 0) mbar_arrive(&ctl.q_rot[q]);
       }
       bool have_rm = false;  // ctl.rm[q][t] holds this row's masks
-      float m_run = -INFINITY, l_run = 0.f;
+      float ref = -INFINITY, l_run = 0.f;  // the row's reference in powers of two, its sum
       // the key tiles that need the mask (tile_needs_mask): those of the block, [jb0, jb1), and
       // those from jm on
       const int jb0 = sd.b0 / kTN, jb1 = sd.blen > 0 ? (sd.b0 + sd.blen + kTN - 1) / kTN : 0;
@@ -549,28 +549,28 @@ __global__ void __launch_bounds__(kPersThreads, 1)
           }
           mask_row(vis64(sd, j * kTN, ctl.rm[q][t]), vis64(sd, j * kTN + 64, ctl.rm[q][t]), sv);
         }
-        // The tile's weights against the reference maximum so far. Their sum stays below
-        // 2^kRescaleLog2 unless the tile's maximum exceeds the reference by more than that in
-        // probability: only then, and before the first finite score, is the maximum formed,
-        // the reference raised to it, the weights computed (again) and O rescaled.
-        float ls, alpha = 1.f;
+        // The tile's weights against the reference so far, the maximum of the row's first tile
+        // with a finite score. Only where their sum comes out at kRescaleMax or more, and before
+        // the first finite score, is the maximum formed and the reference raised beyond it, the
+        // weights are computed (again) and O is rescaled.
+        float ls = 0.f, alpha = 1.f;
         uint32_t pk[32], pk1[32];
         bool rescale = false;
-        bool raise = fresh;
+        bool raise = fresh, over = false;  // over: the second pass, for rows whose sum was
 #pragma unroll 1
         while (true) {
           if (raise) {
-            const float mt = tile_row_max(sv);
-            fresh = __any_sync(0xffffffffu, m_run == -INFINITY && mt == -INFINITY);
-            if (m_run == -INFINITY) {
-              m_run = mt;
-            } else if ((mt - m_run) * sl > kRescaleLog2) {
+            const float top = tile_row_max(sv) * sl;
+            fresh = __any_sync(0xffffffffu, ref == -INFINITY && top == -INFINITY);
+            if (ref == -INFINITY) {
+              ref = top;
+            } else if (!(ls < kRescaleMax) && top > ref) {  // (no other row matters)
               rescale = true;
-              alpha = ex2_approx((m_run - mt) * sl);
-              m_run = mt;
+              alpha = ex2_approx(ref - (top + kRaiseRoom));
+              ref = top + kRaiseRoom;
             }
           }
-          const float mL = m_run == -INFINITY ? 0.f : m_run * sl;
+          const float mL = ref == -INFINITY ? 0.f : ref;
           const uint64_t nmL2 = f2_pack(-mL, -mL);
           uint64_t acc[4] = {0, 0, 0, 0};  // bit pattern 0 = +0.0f
           tile_row_exp<0>(sv, sl2, nmL2, acc, pk);
@@ -579,8 +579,8 @@ __global__ void __launch_bounds__(kPersThreads, 1)
           f2_unpack(f2_add(acc[0], acc[1]), a0, a1);
           f2_unpack(f2_add(acc[2], acc[3]), b0, b1);
           ls = (a0 + a1) + (b0 + b1);
-          if (raise || !__any_sync(0xffffffffu, !(ls < kRescaleMax))) break;
-          raise = true;
+          if (over || !__any_sync(0xffffffffu, !(ls < kRescaleMax))) break;
+          raise = over = true;
         }
         // P_q(n) replaces P_q(n - 1), and O_q may be rescaled, once PV_q(n - 1) has completed
         // (an item's first tile: waited for at the end of the item before)
