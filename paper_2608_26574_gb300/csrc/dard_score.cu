@@ -506,9 +506,10 @@ __device__ __forceinline__ void add_count(const ScoreParams& p, int seq, int sta
   if (p.counts != nullptr) atomicAdd(&p.counts[seq * 3 + state], 1);
 }
 
-// kExtra: the call asks for p_cur, next-step tokens or an in-place state update.
-template <class T, int VPT, bool kExtra>
-__global__ void __launch_bounds__(kScoreThreads, T::W == 4 ? 6 : 5) score_pass1(const __grid_constant__ ScoreParams p) {
+// kExtra: the call asks for p_cur, next-step tokens or an in-place state update. kRegs per thread:
+// what the variant takes without spills, or less where many CTAs run (launch_rows).
+template <class T, int VPT, bool kExtra, int kRegs>
+__global__ void __maxnreg__(kRegs) score_pass1(const __grid_constant__ ScoreParams p) {
   // Launched with programmatic dependent launch after whatever kernel precedes the call
   // (the LM head in a model, the attention kernel in the benchmark): this CTA may already be
   // resident, but it touches no memory before that kernel has completed. Only then may
@@ -914,10 +915,10 @@ cudaError_t launch_fused(const ScoreParams& p, cudaStream_t stream) {
   return cudaLaunchKernelEx(&cfg, score_fused<T, VPT, kExtra>, p);
 }
 
-template <class T, int VPT, bool kExtra, int kCtas>
+template <class T, int VPT, bool kExtra, int kRegs1, int kCtas>
 cudaError_t launch_pair(const ScoreParams& p, cudaStream_t stream) {
   static std::atomic<uint64_t> done1{0}, done2{0};
-  cudaError_t e = allow_wide_clusters(score_pass1<T, VPT, kExtra>, done1);
+  cudaError_t e = allow_wide_clusters(score_pass1<T, VPT, kExtra, kRegs1>, done1);
   if (e == cudaSuccess) e = allow_wide_clusters(score_pass2<T, VPT, kExtra, kCtas>, done2);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -934,7 +935,7 @@ cudaError_t launch_pair(const ScoreParams& p, cudaStream_t stream) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  e = cudaLaunchKernelEx(&cfg, score_pass1<T, VPT, kExtra>, p);
+  e = cudaLaunchKernelEx(&cfg, score_pass1<T, VPT, kExtra, kRegs1>, p);
   if (e != cudaSuccess) return e;
   cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, score_pass2<T, VPT, kExtra, kCtas>, p);
@@ -1017,16 +1018,40 @@ cudaError_t launch_rows(ScoreParams& p, cudaStream_t stream, int per_round) {
     }
     p = keep;
   }
-  // Three CTAs of pass 2 per SM with 80 registers each, or four with 64 and a few spills, by the
-  // CTAs of both passes (about half are pass 2's). Measured (us, bf16 with every output, three
-  // and four): 32 rows of 126464 logits 9.9 and 10.6, 64 of 151936 15.0 and 16.3 (640 CTAs); 64 of
-  // 100000 14.1 and 12.0 (832 CTAs), 1024 of 100000 80.6 and 76.1.
-  if constexpr (kExtra && T::W == 8)
-    if (static_cast<long long>(p.rows) * p.nsplit <= 5ll * sm_count())
-      return launch_pair<T, 4, kExtra, 3>(p, stream);
-  return launch_pair<T, 4, kExtra, 4>(p, stream);
+  // bf16 with end-of-step outputs, by the CTAs of both passes (about half are each pass's).
+  // Pass 1: 56 registers without a spill, or 48 with one where five CTAs per SM matter more. us, with
+  // 56 and 48: 256 rows of 8192 logits 8.9 and 9.9, 32 of 151936 11.7 and 12.5, 64 of 100000 11.8
+  // and 12.4, 128 of 126464 (1024 CTAs) 18.8 and 19.8; 256 of 75776 (1280 CTAs) 25.7 and 24.7, 128
+  // of 151936 25.0 and 23.7.
+  // Pass 2: three CTAs per SM with 80 registers each, or four with 64 and a few spills: 32 rows of
+  // 126464 logits 9.9 and 10.6, 64 of 151936 15.0 and 16.3 (640 CTAs); 64 of 100000 14.1 and 12.0
+  // (832 CTAs), 1024 of 100000 80.6 and 76.1. Rows of one CTA each have no cluster to wait for and
+  // turn sooner: 512 of 4096 11.9 and 12.3, 600 of 8192 13.1 and 12.1, 700 of 4096 14.1 and 13.4.
+  if constexpr (kExtra && T::W == 8) {
+    const long long ctas = static_cast<long long>(p.rows) * p.nsplit, sms = sm_count();
+    if (2 * ctas <= (p.nsplit == 1 ? 7 : 10) * sms)
+      return launch_pair<T, 4, kExtra, 56, 3>(p, stream);
+    if (ctas <= 8 * sms) return launch_pair<T, 4, kExtra, 56, 4>(p, stream);
+  }
+  return launch_pair<T, 4, kExtra, T::W == 4 ? 40 : 48, 4>(p, stream);
 }
 
+}  // namespace
+
+// Whether the launch's one-round clusters leave room for bf16 with end-of-step outputs: about half of
+// them are each pass's, four CTAs fit on an SM, and wide clusters pack the chip less well, so CTAs per
+// SM do not tell. us in one round and in two, by rows over the clusters of pass 1 that fit at once:
+// 1.94 (64 rows of 126464 logits, clusters of 16) 16.3 and 14.9, 1.98 (160 of 50257, 7) 16.3 and 15.2,
+// 2.0 (80 of 100000, 13) 16.3 and 14.9, 2.1 (128 of 70000, 9) 17.1 and 15.0; while at 1.73 (128 of
+// 65536, 8) 13.3 and 14.8, (256 of 32000, 4) 14.1 and 15.3.
+namespace {
+bool one_round_fits(const ScoreParams& p) {
+  static std::atomic<uint64_t> done{0};
+  const auto kernel = score_pass1<Bf16, 4, true, 56>;
+  if (allow_wide_clusters(kernel, done) != cudaSuccess) return true;
+  const int n = max_active_clusters(kernel, p.nsplit);
+  return n == 0 || 20ll * p.rows < 37ll * n;
+}
 }  // namespace
 
 dard_status launch_score(const dard_score_args& a, ScoreParams& p, cudaStream_t stream,
@@ -1035,12 +1060,15 @@ dard_status launch_score(const dard_score_args& a, ScoreParams& p, cudaStream_t 
   const int W = bf16 ? 8 : 4;
   const int per_round = kScoreThreads * 4 * W;
   set_split(p, per_round, split_cap(p.rows));
+  const bool extra = p.p_cur != nullptr || p.tokens != nullptr || p.state_in_place ||
+                     p.entropy != nullptr || p.margin != nullptr || p.order_key != nullptr;
   // CTAs of one round only while the launch's fit at once (four to five per SM, about half of the
   // rows being each pass's): a second wave of them costs its merges again. Two rounds, measured
   // against one: 128 rows of 100000 bf16 logits 16.5 -> 13.4 us, 256 of 50000 16.6 -> 14.7, 128 of
   // 50000 fp32 14.4 -> 11.5; with room for all (128 of 50000 bf16) one round stays.
   if (p.chunk == per_round && p.nsplit > 1 &&
-      static_cast<long long>(p.rows) * p.nsplit > 8ll * sm_count())
+      (static_cast<long long>(p.rows) * p.nsplit > 8ll * sm_count() ||
+       (bf16 && extra && !one_round_fits(p))))
     set_split(p, per_round, (p.nsplit + 1) / 2);
 
   char* ws = static_cast<char*>(a.workspace);
@@ -1065,8 +1093,6 @@ dard_status launch_score(const dard_score_args& a, ScoreParams& p, cudaStream_t 
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && p.rows > 0) {
-    const bool extra = p.p_cur != nullptr || p.tokens != nullptr || p.state_in_place ||
-                       p.entropy != nullptr || p.margin != nullptr || p.order_key != nullptr;
     if (extra) e = bf16 ? launch_rows<Bf16, true>(p, stream, per_round)
                         : launch_rows<F32, true>(p, stream, per_round);
     else e = bf16 ? launch_rows<Bf16, false>(p, stream, per_round)
