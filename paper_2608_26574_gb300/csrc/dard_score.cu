@@ -675,8 +675,10 @@ __device__ __forceinline__ void red_release_gpu(uint32_t* p, uint32_t v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// Four CTAs per SM, as every row's cluster has to fit at once: with the 80 registers that it would
+// take instead of 64 the splits shrink (256 rows of 126464 bf16 logits 46.3 us, so 34.6).
 template <class T, int VPT, bool kExtra>
-__global__ void __launch_bounds__(kScoreThreads) score_fused(const __grid_constant__ ScoreParams p) {
+__global__ void __launch_bounds__(kScoreThreads, 4) score_fused(const __grid_constant__ ScoreParams p) {
   // Launched as a programmatic dependent of whatever kernel precedes the call: nothing is
   // read before that kernel (the logits' producer, or the previous call that leaves the
   // counters at zero) has completed.
@@ -999,9 +1001,8 @@ void set_split(ScoreParams& p, int per_round, int cap) {
 // The two PDL-chained passes; with DARD_SCORE_PATH=fused, the one-launch kernel instead when
 // every row's cluster fits on the device at once (its M rows wait for C rows of the same
 // launch), with as many CTAs per row as allows that. Measured on GB300 (CUDA-graph timing,
-// one call per input set): the passes take 8.3 us on the 8B block, 13.5 us on the GQA block,
-// 25 us on the multimodal batch; the one launch 11.9, 18.4 and 34 us (10.4, 16.2 with no
-// counts requested). The pass boundary is a completed grid, which the hardware signals
+// one call per input set, with counts): the passes take 8.2 us on the 8B block, 12.4 us on the GQA
+// block, 25.6 us on the multimodal batch; the one launch 12.4, 17.5 and 34.6 us. The pass boundary is a completed grid, which the hardware signals
 // sooner than the counters in L2 that the one launch polls.
 template <class T, bool kExtra>
 cudaError_t launch_rows(ScoreParams& p, cudaStream_t stream, int per_round) {
