@@ -168,6 +168,10 @@ typedef enum { DARD_ROPE_INTERLEAVED = 0, DARD_ROPE_HALF = 1 } dard_rope_style;
  * library picks the one a cost model of the batch (query tiles, key tiles, SM count) predicts
  * to be faster; the environment variable DARD_ATTN_TC=1 or 2 forces one of them (results
  * agree within rounding).
+ * A key that a row does not see has weight 0. With F32 nothing else of it reaches the row, whatever
+ * k and v hold there. With BF16 the tensor cores multiply its v row by that 0, and the last key
+ * tile of a sequence reaches up to 127 rows into the next one: v must be finite in every row of the
+ * call (k need not be where no row sees it).
  * Errors: DARD_ERR_NULL (also: k_rope NULL with rope_theta > 0), _SHAPE, _VALUE (scale < 0
  * or not finite; rope_theta neither 0 nor a finite value >= 1; rope_style not a
  * dard_rope_style), _UNSUPPORTED, _ALIGN, _CUDA. */
@@ -323,7 +327,7 @@ dard_status dard_score_and_transition_noalloc(const dard_score_args* args, void*
  * alignment of the type (16-byte accesses where the rows allow them); arithmetic in fp32.
  *   dard_add_rmsnorm  s = x + add (add NULL: x), rounded to dtype; sum = s (sum NULL: not
  *                     stored); out = s / sqrt(mean(s^2) + eps) per row. sum and out may each
- *                     be x or add.
+ *                     be x or add, but not the same buffer.
  *   dard_swiglu       out = a / (1 + exp(-a)) * b over n elements; out may be a or b.
  * Errors: DARD_ERR_NULL, _SHAPE, _VALUE, _ALIGN, _CUDA. */
 dard_status dard_add_rmsnorm(const void* x, const void* add, void* sum, void* out, int32_t rows,

@@ -52,7 +52,7 @@ const char* dard_status_string(dard_status s) {
 
 const char* dard_last_error(void) { return g_err; }
 
-int32_t dard_version(void) { return 20100; }
+int32_t dard_version(void) { return 20200; }
 
 }  // extern "C"
 

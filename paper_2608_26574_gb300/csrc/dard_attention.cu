@@ -43,8 +43,11 @@
 //   S_q(j + 1) in the pipe, since the one S buffer's turnaround is the critical path and the
 //   pipe runs two threads' products interleaved (231 us); no maximum and no mask arithmetic on
 //   the common tile (217 us).
-// Both keep a per-row running maximum and rescale O in TMEM only when the maximum grows by
-// more than a factor 2^8 (the exponentials stay bounded by 2^8 otherwise).
+//   (The times here and in choose_tc are of single launches; back to back for seconds the board is
+//   at its power limit, and the two larger workloads take 245 and 849 us.)
+// Both take a row's weights against a reference and rescale O in TMEM only when it moves: in attn_tc1
+// a running maximum that moves when it grows by more than a factor 2^8, in attn_tc2 that of the first
+// tile until a tile's sum reaches 2^8 (kRaiseRoom). The weights stay below 2^8.
 // fp32 paths: attn_simt (dard_attention_simt.cu) and attn_f32 (dard_attention_f32.cu), CUDA
 // cores, the same mask logic.
 #include <algorithm>
@@ -494,31 +497,6 @@ __global__ void __launch_bounds__(kTc1Threads, 1)
 }
 
 
-// The visibility bits applied to a row's 128 scores (vis0: keys 0-63, vis1: 64-127): a hidden
-// key becomes -inf.
-__device__ __forceinline__ void mask_row(uint64_t vis0, uint64_t vis1, uint32_t (&sv)[128]) {
-#pragma unroll
-  for (int k = 0; k < 128; ++k) {
-    const uint64_t vis = k < 64 ? vis0 : vis1;
-    sv[k] = ((vis >> (k & 63)) & 1ull) ? sv[k] : 0xff800000u;  // -inf
-  }
-}
-
-__device__ __forceinline__ float tile_row_max(const uint32_t (&sv)[128]) {
-  float mx[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e)
-    mx[e] = fmax3(__uint_as_float(sv[e]), __uint_as_float(sv[8 + e]), __uint_as_float(sv[16 + e]));
-#pragma unroll
-  for (int k = 24; k < 128; k += 16) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e)
-      mx[e] = k + 8 + e < 128 ? fmax3(mx[e], __uint_as_float(sv[k + e]), __uint_as_float(sv[k + 8 + e]))
-                              : fmaxf(mx[e], __uint_as_float(sv[k + e]));
-  }
-  return fmaxf(fmax3(mx[0], mx[1], mx[2]), fmax3(fmax3(mx[3], mx[4], mx[5]), mx[6], mx[7]));
-}
-
 // P = 2^(s * sl - mL) of the row's 128 scores as bf16 pairs, and their sum: of the rounded
 // values, so that the output is a convex combination of V rows with exactly the weights the
 // PV product uses.
@@ -557,7 +535,7 @@ struct __align__(16) Tc2Ctl {
   // issuer of PV has taken phase j of its slot before phase j + 4 completes (and before
   // j + 3: three slots would do).
   uint64_t pv_go[kQT][kPvGo];
-  uint64_t pv_done[kQT];  // PV_q(j) completed: S_q's columns may take S_q(j + 1)
+  uint64_t pv_done[kQT];  // PV_q(j) completed: P_q(j + 1) may replace P_q(j), O_q be rescaled
   uint64_t o_full[kQT];   // the last PV_q completed
   uint64_t drained;       // every product both issuers launched has completed (two commits)
   uint32_t tmem_base;
@@ -836,7 +814,7 @@ __global__ void __launch_bounds__(kTc2Threads, 1)
                     : mbar_wait(&ctl.s_full[q], j & 1, wlim));
       if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
       tc_fence_after();
-      // the tile's 128 scores of this row in registers, and their maximum
+      // the tile's 128 scores of this row in registers
       uint32_t sv[128];
 #pragma unroll
       for (int c = 0; c < 4; ++c)
@@ -1009,21 +987,6 @@ int choose_tc(const AttnParams& p, int sms, int forced, bool* persist) {
   return kernel;
 }
 
-// attn_tc2's register split assumes a launch allocation of kTc2LaunchRegs per thread; with
-// any other, setmaxnreg.inc would wait for registers that never come. A build that allocated
-// otherwise is refused before its first launch (checked once per instantiation).
-template <class F>
-cudaError_t check_tc2_regs(F* kernel, std::atomic<int>& state) {
-  const int known = state.load(std::memory_order_acquire);
-  if (known != 0) return known == 1 ? cudaSuccess : cudaErrorInvalidDeviceFunction;
-  cudaFuncAttributes fa;
-  const cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-  if (e != cudaSuccess) return e;
-  const bool ok = fa.numRegs == static_cast<int>(kTc2LaunchRegs);
-  state.store(ok ? 1 : 2, std::memory_order_release);
-  return ok ? cudaSuccess : cudaErrorInvalidDeviceFunction;
-}
-
 template <int D>
 cudaError_t launch_tc(const AttnParams& p, int kernel, cudaStream_t stream) {
   static std::atomic<uint64_t> attr1_done{0}, attr2_done{0}, attr2r_done{0};
@@ -1037,11 +1000,11 @@ cudaError_t launch_tc(const AttnParams& p, int kernel, cudaStream_t stream) {
     static std::atomic<int> regs2{0}, regs2r{0};
     const AttnLaunch L(p.total_pairs, kTc2Threads, smem, stream, 1, p.rope != 0);
     if (p.rope) {
-      cudaError_t e = check_tc2_regs(attn_tc2<D, true>, regs2r);
+      cudaError_t e = check_launch_regs(attn_tc2<D, true>, kTc2LaunchRegs, regs2r);
       if (e == cudaSuccess) e = ensure_smem_attr(attn_tc2<D, true>, smem, attr2r_done);
       return e != cudaSuccess ? e : cudaLaunchKernelEx(&L.cfg, attn_tc2<D, true>, p, mq, mk, mv);
     }
-    cudaError_t e = check_tc2_regs(attn_tc2<D, false>, regs2);
+    cudaError_t e = check_launch_regs(attn_tc2<D, false>, kTc2LaunchRegs, regs2);
     if (e == cudaSuccess) e = ensure_smem_attr(attn_tc2<D, false>, smem, attr2_done);
     return e != cudaSuccess ? e : cudaLaunchKernelEx(&L.cfg, attn_tc2<D, false>, p, mq, mk, mv);
   }

@@ -32,15 +32,13 @@
 // (239 us with the split above, as without batches); O stored by each row's own thread with
 // 32-byte stores (ragged batch 790 -> 822 us).
 #include <algorithm>
-#include <cstdio>
-#include <cstdlib>
 
 #include "dard_attn_common.cuh"
 
 namespace dard {
 namespace {
 
-constexpr int kPersThreads = 384;  // 2 x 4 softmax warps, TMA producer, S and PV issuers, spare
+constexpr int kPersThreads = 384;  // 2 x 4 softmax warps, TMA producer, S and PV issuers, item decoder
 constexpr int kQT = 2;    // query tiles per work item at most (one sequence and K/V head)
 constexpr int kNK = 2;    // TMA stages for K
 constexpr int kNV = 2;    // TMA stages for V
@@ -52,38 +50,13 @@ constexpr int kWMma = kWProd + 1;  // warp 9: TMEM allocator and S issuer
 constexpr int kWPv = kWProd + 2;   // warp 10: PV issuer
 constexpr int kWItem = kWProd + 3;  // warp 11: item decoder
 // Register split (setmaxnreg): the launch gives 384 threads 168 registers each; the
-// warpgroup of warps 8-11 (producer, issuers, spare) drops to 40 and the two softmax
+// warpgroup of warps 8-11 (producer, issuers, decoder) drops to 40 and the two softmax
 // warpgroups rise to 232, so that a thread holds its row's 128 scores and 64 words of
 // weights at once: 128 x 40 + 256 x 232 = 384 x 168.
 constexpr uint32_t kPersLaunchRegs = 168, kPersSideRegs = 40, kPersSoftmaxRegs = 232;
 static_assert(128 * kPersSideRegs + 256 * kPersSoftmaxRegs == kPersThreads * kPersLaunchRegs,
               "the register shares must add up to the launch's registers");
 static_assert(kPersThreads * kPersLaunchRegs <= 65536, "one CTA per SM");
-
-// The visibility bits applied to a row's 128 scores (vis0: keys 0-63, vis1: 64-127): a hidden
-// key becomes -inf.
-__device__ __forceinline__ void mask_row(uint64_t vis0, uint64_t vis1, uint32_t (&sv)[128]) {
-#pragma unroll
-  for (int k = 0; k < 128; ++k) {
-    const uint64_t vis = k < 64 ? vis0 : vis1;
-    sv[k] = ((vis >> (k & 63)) & 1ull) ? sv[k] : 0xff800000u;  // -inf
-  }
-}
-
-__device__ __forceinline__ float tile_row_max(const uint32_t (&sv)[128]) {
-  float mx[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e)
-    mx[e] = fmax3(__uint_as_float(sv[e]), __uint_as_float(sv[8 + e]), __uint_as_float(sv[16 + e]));
-#pragma unroll
-  for (int k = 24; k < 128; k += 16) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e)
-      mx[e] = k + 8 + e < 128 ? fmax3(mx[e], __uint_as_float(sv[k + e]), __uint_as_float(sv[k + 8 + e]))
-                              : fmaxf(mx[e], __uint_as_float(sv[k + e]));
-  }
-  return fmaxf(fmax3(mx[0], mx[1], mx[2]), fmax3(fmax3(mx[3], mx[4], mx[5]), mx[6], mx[7]));
-}
 
 // P = 2^(s * sl - mL) of keys 64 hh .. 64 hh + 63 of the row's scores as bf16 pairs, and their
 // sum: of the rounded values, so that the output is a convex combination of V rows with exactly
@@ -107,7 +80,7 @@ __device__ __forceinline__ void tile_row_exp(const uint32_t (&sv)[128], uint64_t
 // tiles [0, nk[q]), and its sequence's layout. nq = 0 ends the CTA's items.
 struct __align__(16) TcItem {
   SeqDesc sd;
-  int32_t seq, g, nq, first;  // first: the sequence's first item (reports bad states once)
+  int32_t g, nq, first;  // first: the sequence's first item (reports bad states once)
   int32_t r[kQT], h[kQT], nk[kQT], n_kt;  // n_kt: the larger of nk
 };
 
@@ -136,7 +109,6 @@ struct __align__(16) PersistCtl {
                           // last key tile O_q is final
   uint64_t drained;       // every product both issuers launched has completed (two commits)
   uint32_t tmem_base;
-  int32_t abort;
   TcItem item[kItems];
   BlockInfo bi[kItems];   // the block of each item's sequence
   RowMasks rm[kQT][kBM];  // each row's masks, read on the tiles that need them
@@ -149,8 +121,7 @@ constexpr size_t persist_smem_bytes() {
   return 1024 + (kQT + kNK + kNV) * static_cast<size_t>(kTN) * D * 2 + sizeof(PersistCtl);
 }
 
-__device__ __forceinline__ void flag_timeout(const AttnParams& p, PersistCtl& ctl) {
-  ctl.abort = 1;
+__device__ __forceinline__ void flag_timeout(const AttnParams& p) {
   if (p.status) atomicOr(p.status, DARD_STATUS_TIMEOUT);
 }
 
@@ -177,7 +148,6 @@ __device__ __forceinline__ TcItem tc_item(const AttnParams& p, int k) {
   const int rows = sd.n_orig + sd.slen;
   const int local = lo == 0 ? w : w - p.item_prefix[lo];
   it.sd = sd;
-  it.seq = seq;
   it.first = local == 0;
   int nq, r0, r1, nk0, nk1;
   if (p.by_group) {
@@ -292,7 +262,6 @@ __global__ void __launch_bounds__(kPersThreads, 1)
       mbar_init(&ctl.v_empty[b], 1);
     }
     mbar_init(&ctl.drained, 2);
-    ctl.abort = 0;
     fence_barrier_init();
     tma_prefetch_desc(&tmv);
   }
@@ -359,7 +328,7 @@ __global__ void __launch_bounds__(kPersThreads, 1)
         }
         done_with(k);
       }
-      if (!ok) flag_timeout(p, ctl);
+      if (!ok) flag_timeout(p);
       // Every copy issued lands before shared memory is released (after a normal run they all
       // have: the waits return at once): the latest use of each stage (earlier uses landed
       // before their stage was reused). A copy the test hook dropped was never issued.
@@ -429,7 +398,7 @@ __global__ void __launch_bounds__(kPersThreads, 1)
         __syncwarp();
       }
     }
-    if (!ok && lane == 0) flag_timeout(p, ctl);
+    if (!ok && lane == 0) flag_timeout(p);
     if (elect_one()) mma_commit(&ctl.drained);  // completes once every S product issued has
     __syncwarp();
   } else if (warp == kWPv) {
@@ -479,7 +448,7 @@ __global__ void __launch_bounds__(kPersThreads, 1)
         __syncwarp();
       }
     }
-    if (!ok && lane == 0) flag_timeout(p, ctl);
+    if (!ok && lane == 0) flag_timeout(p);
     if (elect_one()) mma_commit(&ctl.drained);  // completes once every PV product issued has
     __syncwarp();
   } else if (warp < kWProd) {
@@ -656,7 +625,7 @@ __global__ void __launch_bounds__(kPersThreads, 1)
       // the reads of O come before the first P_q of the next item, which lets PV_q write O
       tc_fence_before();
     }
-    if (!ok && lane == 0) flag_timeout(p, ctl);
+    if (!ok && lane == 0) flag_timeout(p);
   } else {
     // ------------------------------------------------------------ item decoder
     // One warp decodes the items (searches and cold parameter reads, about 1000 cycles) and
@@ -679,13 +648,13 @@ __global__ void __launch_bounds__(kPersThreads, 1)
       if (lane == 0) mbar_arrive(&ctl.bi_full[b]);
       __syncwarp();
     }
-    if (!ok && lane == 0) flag_timeout(p, ctl);
+    if (!ok && lane == 0) flag_timeout(p);
   }
   tc_fence_before();
   __syncthreads();
   if (warp == kWMma) {
     // no product is still writing TMEM (both issuers committed `drained` last)
-    if (lane == 0 && !mbar_wait(&ctl.drained, 0, wlim)) flag_timeout(p, ctl);
+    if (lane == 0 && !mbar_wait(&ctl.drained, 0, wlim)) flag_timeout(p);
     __syncwarp();
     tc_fence_after();
     tmem_dealloc<kTmemCols>(ctl.tmem_base);
@@ -693,21 +662,6 @@ __global__ void __launch_bounds__(kPersThreads, 1)
 }
 
 // ---------------------------------------------------------------- host side
-
-// The register split assumes a launch allocation of kPersLaunchRegs per thread; with any
-// other, setmaxnreg.inc would wait for registers that never come. A build that allocated
-// otherwise is refused before its first launch (checked once per instantiation).
-template <class F>
-cudaError_t check_regs(F* kernel, std::atomic<int>& state) {
-  const int known = state.load(std::memory_order_acquire);
-  if (known != 0) return known == 1 ? cudaSuccess : cudaErrorInvalidDeviceFunction;
-  cudaFuncAttributes fa;
-  const cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
-  if (e != cudaSuccess) return e;
-  const bool ok = fa.numRegs == static_cast<int>(kPersLaunchRegs);
-  state.store(ok ? 1 : 2, std::memory_order_release);
-  return ok ? cudaSuccess : cudaErrorInvalidDeviceFunction;
-}
 
 template <int D, bool kRope>
 cudaError_t launch(const AttnParams& p, cudaStream_t stream) {
@@ -719,7 +673,7 @@ cudaError_t launch(const AttnParams& p, cudaStream_t stream) {
       !make_map(&mv, p.v, p.hkv, D, p.total_rows, kTN))
     return cudaErrorInvalidValue;
   const size_t smem = persist_smem_bytes<D>();
-  cudaError_t e = check_regs(attn_persist<D, kRope>, regs);
+  cudaError_t e = check_launch_regs(attn_persist<D, kRope>, kPersLaunchRegs, regs);
   if (e == cudaSuccess) e = ensure_smem_attr(attn_persist<D, kRope>, smem, attr_done);
   if (e != cudaSuccess) return e;
   const AttnLaunch L(persist_ctas(p), kPersThreads, smem, stream, 1, kRope);

@@ -1,5 +1,5 @@
-// dard_attn_common.cuh - pieces shared by the attention kernels (dard_attention.cu,
-// dard_attention_pair.cu): the per-CTA copy of the current block, the in-kernel mask of
+// dard_attn_common.cuh - pieces shared by the attention kernels (dard_attention.cu and the
+// dard_attention_*.cu): the per-CTA copy of the current block, the in-kernel mask of
 // Sec. 3.2 (which copy, x^j or s^j, a query attends for every position j), the ragged
 // work decoding, and the host helpers for tensor maps and kernel attributes.
 #pragma once
@@ -342,6 +342,31 @@ constexpr int kTN = 128;  // keys per tile of the tensor-core path
 constexpr int kL2Ahead = 4;  // K/V tiles the CTA-pair kernel prefetches into L2 ahead of its
                               // TMA loads (the one-CTA kernel: none, measured faster)
 
+// The visibility bits applied to a row's 128 scores (vis0: keys 0-63, vis1: 64-127): a hidden
+// key becomes -inf.
+__device__ __forceinline__ void mask_row(uint64_t vis0, uint64_t vis1, uint32_t (&sv)[128]) {
+#pragma unroll
+  for (int k = 0; k < 128; ++k) {
+    const uint64_t vis = k < 64 ? vis0 : vis1;
+    sv[k] = ((vis >> (k & 63)) & 1ull) ? sv[k] : 0xff800000u;  // -inf
+  }
+}
+
+__device__ __forceinline__ float tile_row_max(const uint32_t (&sv)[128]) {
+  float mx[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e)
+    mx[e] = fmax3(__uint_as_float(sv[e]), __uint_as_float(sv[8 + e]), __uint_as_float(sv[16 + e]));
+#pragma unroll
+  for (int k = 24; k < 128; k += 16) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      mx[e] = k + 8 + e < 128 ? fmax3(mx[e], __uint_as_float(sv[k + e]), __uint_as_float(sv[k + 8 + e]))
+                              : fmaxf(mx[e], __uint_as_float(sv[k + e]));
+  }
+  return fmaxf(fmax3(mx[0], mx[1], mx[2]), fmax3(fmax3(mx[3], mx[4], mx[5]), mx[6], mx[7]));
+}
+
 static_assert(kTN == kKeyTile, "one key-tile width for the kernels and the planner");
 
 __device__ __forceinline__ bool tile_needs_mask(const SeqDesc& sd, int kt0) {
@@ -472,6 +497,21 @@ struct AttnLaunch {
   AttnLaunch(const AttnLaunch&) = delete;
   AttnLaunch& operator=(const AttnLaunch&) = delete;
 };
+
+// A register split (setmaxnreg) assumes a launch allocation of `regs` per thread; with any other,
+// setmaxnreg.inc would wait for registers that never come. A build that allocated otherwise is
+// refused before its first launch (checked once per instantiation).
+template <class F>
+cudaError_t check_launch_regs(F* kernel, uint32_t regs, std::atomic<int>& state) {
+  const int known = state.load(std::memory_order_acquire);
+  if (known != 0) return known == 1 ? cudaSuccess : cudaErrorInvalidDeviceFunction;
+  cudaFuncAttributes fa;
+  const cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess) return e;
+  const bool ok = fa.numRegs == static_cast<int>(regs);
+  state.store(ok ? 1 : 2, std::memory_order_release);
+  return ok ? cudaSuccess : cudaErrorInvalidDeviceFunction;
+}
 
 // SMs of the current device, 0 without one (looked up once per device).
 int device_sms() {

@@ -96,7 +96,7 @@ class DLLM:
                                     rope_theta=cfg.rope_base,
                                     rope_style=B.DARD_ROPE_INTERLEAVED)
         # Norms (with the residual add before them) and gates are one launch each: as tensor
-        # operations they were 30 of the launches of a layer, and launching took most of the
+        # operations they were 18 of the launches of a layer, and launching took most of the
         # time of a forward pass (two layers of d_model 1024, 2688 rows).
         delta = None  # what the layer before adds to h
         for L in self.layers:
