@@ -882,10 +882,10 @@ cudaError_t allow_wide_clusters(F* kernel, std::atomic<uint64_t>& done) {
   return e;
 }
 
-// Clusters of nsplit CTAs of this kernel that fit on the current device at once (cached
-// per device and cluster size).
-template <class K>
-int max_active_clusters(K* kernel, int nsplit) {
+// Clusters of nsplit CTAs of this kernel that fit on the current device at once (cached per kernel,
+// by its value: all of them have one type; per device and cluster size).
+template <auto kKernel>
+int max_active_clusters(int nsplit) {
   static std::atomic<int> cache[64][kScoreMaxSplit + 1];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || nsplit < 1 ||
@@ -903,7 +903,7 @@ int max_active_clusters(K* kernel, int nsplit) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n <= 0) {
+  if (cudaOccupancyMaxActiveClusters(&n, kKernel, &cfg) != cudaSuccess || n <= 0) {
     cudaGetLastError();
     return 0;
   }
@@ -1026,7 +1026,7 @@ cudaError_t launch_rows(ScoreParams& p, cudaStream_t stream, int per_round) {
     const ScoreParams keep = p;
     for (int cap = p.nsplit; cap >= 1; --cap) {
       set_split(p, per_round, cap);
-      if (max_active_clusters(score_fused<T, 4, kExtra>, p.nsplit) >= p.rows)
+      if (max_active_clusters<score_fused<T, 4, kExtra>>(p.nsplit) >= p.rows)
         return launch_fused<T, 4, kExtra>(p, stream);
       cap = p.nsplit;  // the next smaller split
     }
@@ -1061,9 +1061,9 @@ cudaError_t launch_rows(ScoreParams& p, cudaStream_t stream, int per_round) {
 namespace {
 bool one_round_fits(const ScoreParams& p) {
   static std::atomic<uint64_t> done{0};
-  const auto kernel = score_pass1<Bf16, 4, true, 56>;
-  if (allow_wide_clusters(kernel, done) != cudaSuccess) return true;
-  const int n = max_active_clusters(kernel, p.nsplit);
+  constexpr auto kKernel = score_pass1<Bf16, 4, true, 56>;
+  if (allow_wide_clusters(kKernel, done) != cudaSuccess) return true;
+  const int n = max_active_clusters<kKernel>(p.nsplit);
   return n == 0 || 20ll * p.rows < 37ll * n;
 }
 }  // namespace
