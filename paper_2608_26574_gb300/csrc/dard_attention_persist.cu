@@ -24,10 +24,12 @@
 // (attn_tc2, forced, the same build otherwise): 32 sequences of 500 to 2300 rows 811 -> 759 us,
 // 8 of 1248 rows 173 -> 165 us, a GQA sequence of 5184 rows 217 -> 221 us; a launch of at most
 // one item per SM has nothing to hide and its start is later (8B layer 15.4 -> 17.7 us): those
-// stay with attn_tc1 and attn_tc2.
+// stay with attn_tc1 and attn_tc2. (Single launches; back to back for seconds the board is at its
+// power limit, and the first and the last take 845 and 243 us.)
 //
-// Tried and slower: both tile slots on a lone query tile, every other key tile each, merged at
-// the end (the loop's code got worse: GQA 221 -> 240 us, a lone-tile launch 14.7 -> 16.4 us);
+// Tried and slower: the rows of a last V tile that belong to the next sequence cleared, so that a
+// NaN there stays out (24 sequences of 264 rows 91.0 us, by the PV issuer 94.5, by warp 11 100.4);
+// both tile slots on a lone query tile, every other key tile each, merged at the end (the loop's code got worse: GQA 221 -> 240 us, a lone-tile launch 14.7 -> 16.4 us);
 // P stored and handed over in two halves (226 us); the exponentials in explicit batches of 16
 // (239 us with the split above, as without batches); O stored by each row's own thread with
 // 32-byte stores (ragged batch 790 -> 822 us).

@@ -128,10 +128,10 @@ __device__ __forceinline__ uint4 load_vec(const char* row, int e0, int c1) {
 // the position of the maximum only the vector that holds it (its first element's index and its
 // data): the element within it is looked up once, at the end (winner_index). Tracking the
 // vector takes one comparison per vector where tracking the element took one per value, and
-// the passes over many bf16 rows are bound by
-// their instructions as much as by memory (1024 rows of 126464 bf16 logits, 388 MB: 75.9 -> 72.0
-// us; one block with every end-of-step output 10.4 -> 9.5 us). fp32 rows: see fold_round. Streaming the rounds through shared
-// memory by bulk copies instead, up to 192 KB in flight on an SM, measured no faster (71.4 us).
+// the passes over many bf16 rows are bound by their instructions as much as by memory (1024 rows of
+// 126464 bf16 logits, 388 MB: 76.3 -> 71.8 us; one block with every end-of-step output 10.7 -> 10.0).
+// fp32 rows: see fold_round. Streaming the rounds through shared memory by bulk copies instead, up to
+// 192 KB in flight on an SM, measured no faster (71.4 us).
 template <int kRaw>  // 16-byte vectors of logits behind a vector of scored values
 struct Run {
   float m, s;      // maximum; sum of 2^(x log2 e - reference(m)), of exp(x - m) once merged
