@@ -192,8 +192,8 @@ dard_status dard_attention_kernel(const dard_attn_args* args, int32_t* kernel);
  * launching anything (an interface addition: the paper has no counterpart). The arguments
  * go through the same host validation as dard_step_attention and fail with the same codes.
  *   kernel              as dard_attention_kernel (0: no query rows, nothing launched)
- *   ctas                CTAs of the launch (kernels 1 and 2: at most one per SM, persistent
- *                       beyond one wave; the CTA-pair kernel: two per cluster, as many
+ *   ctas                CTAs of the launch (kernels 1 and 2: one per tile or pair of tiles up to a
+ *                       few waves, where that is cheaper, else at most one per SM, persistent; the CTA-pair kernel: two per cluster, as many
  *                       clusters as fit on the current device, or SMs / 2 without one; fp32:
  *                       four per 128-row query tile and head while those that hold query rows
  *                       are at most one per SM (without a device: while all are at most 148),

@@ -9,7 +9,7 @@
 // shadow keys or the ragged end of the sequence.
 //
 // bf16 paths (tcgen05 MMAs with fp32 accumulators in TMEM, K/V tiles of 128 keys by TMA),
-// one CTA per SM, chosen per call by a cost model (choose_tc); launches of more than one wave
+// one CTA per SM, chosen per call by a cost model (choose_tc); most launches of more than one wave
 // run attn_persist (dard_attention_persist.cu) instead:
 //
 // attn_tc1: 128 query rows of one (sequence, head); 11 warps:
@@ -943,7 +943,8 @@ __global__ void __launch_bounds__(kTc2Threads, 1)
 //      last tile 14000 + 1700 kt);
 //   more than that: attn_persist over items of any two consecutive (tile, head) units of a K/V
 //      head's group (1) or of pairs of a head's tiles (2): 7000 + 2300 kt an item (a lone
-//      tile 7000 + 2000 kt) spread over the SMs, plus half an item of tail and 12000 to start.
+//      tile 7000 + 2000 kt) spread over the SMs, plus half an item of tail and 12000 to start;
+//      but up to three waves of attn_tc2's CTAs: few_waves().
 // Measured, us (8B layer, its prefix-cached variant, GQA sequence, its variant, ragged batch):
 // attn_tc1 22.8, 12.4, 301, 76, 1168; attn_tc2 15.4, 14.6, 217, 54, 811; attn_persist 17.7,
 // 14.7, 221, 58, 759. Equal costs go to 2: the two ways differ only where a group of heads or
@@ -963,6 +964,92 @@ struct TcEstimate {
   }
 };
 
+constexpr int kMaxWaves = 3;  // few_waves: of attn_tc1's or attn_tc2's CTAs
+
+// Work items by cost, and the longest share of one SM where they go out in rows of `sms`, longest
+// first, in alternating direction: attn_persist's order, and about that in which SMs become free.
+struct TcClasses {
+  struct Class {
+    double cost;
+    long long n;
+  } c[2 * DARD_MAX_SEQS];
+  int m = 0;
+  long long items = 0;
+  void add(long long n, double cost) {
+    if (n <= 0) return;
+    items += n;
+    if (m > 0 && c[m - 1].cost == cost) c[m - 1].n += n;
+    else c[m++] = {cost, n};
+  }
+  double share(int sms) {
+    std::sort(c, c + m, [](const Class& a, const Class& b) { return a.cost > b.cost; });
+    const long long rounds = (items + sms - 1) / sms, rem = items - (rounds - 1) * sms;
+    if (rounds > 8) {
+      double total = 0;
+      for (int i = 0; i < m; ++i) total += c[i].cost * static_cast<double>(c[i].n);
+      return total / sms + 0.5 * c[0].cost;
+    }
+    double best = 0;
+    // the SMs at the ends of a row and on either side of the last row's end
+    for (const long long b : {0ll, sms - 1ll, rem - 1, std::min<long long>(rem, sms - 1), sms - rem,
+                              std::max(sms - rem - 1, 0ll)}) {
+      double sum = 0;
+      long long below = 0;  // items of the classes before i
+      int i = 0;
+      for (long long k = 0; k < rounds; ++k) {
+        const long long at = k * sms + ((k & 1) ? sms - 1 - b : b);
+        while (i < m && below + c[i].n <= at) below += c[i++].n;
+        if (i < m) sum += c[i].cost;
+      }
+      best = std::max(best, sum);
+    }
+    return best;
+  }
+};
+
+// The cheapest of attn_tc1 and attn_tc2 in up to three waves and attn_persist in either way. Within
+// few waves the items' granularity decides, not their sum, and attn_persist's later start counts.
+// Costs fitted to 880 CUDA-graph timings of the four over 220 batches of 1 to 40 sequences (9 %
+// rms); what it picks takes 0.7 % more than the best of the four, attn_persist alone 4 %. us
+// (attn_tc1, attn_tc2, attn_persist): 3 sequences of 3 tiles, 32 heads 18.3, 17.7, 22.4; 2 of 5 tiles
+// 29.3, 22.2, 26.2; 3 of 6 tiles, 28 / 4 heads 42.3, 27.4, 30.7; 10 of one query tile against 25 to 28
+// key tiles, 16 heads of 64, with RoPE 63.2, 75.1, 76.0; 26 of 2 tiles, 32 heads, with RoPE (six
+// waves) 113.6, 86.7, 79.5.
+int few_waves(const AttnParams& p, int sms, bool* persist) {
+  const bool d128 = p.head_dim == 128, rope = p.rope != 0;
+  const double r1 = rope ? 2900 : 0, r2 = rope ? 5300 : 0, rp = rope ? 6000 : 0;
+  TcClasses t1, t2, p1, p2;
+  const long long per_group = p.hq / p.hkv;
+  for (int s = 0; s < p.num_seqs; ++s) {
+    const SeqDesc& sd = p.seq[s];
+    const double kt = (sd.n_orig + sd.slen + kTN - 1) / kTN;
+    const long long n = sd.n_qtiles, units = n * per_group;
+    const double item = 10600 + (d128 ? 2800 : 2450) * kt + rp;
+    const double lone = 8300 + (d128 ? 2500 : 1950) * kt + rp;
+    t1.add(n * p.hq, 11000 + (d128 ? 1900 : 1350) * kt + r1);
+    t2.add(n / 2 * p.hq, 12000 + (d128 ? 2650 : 2450) * kt + r2);
+    t2.add(n % 2 * p.hq, 9400 + (d128 ? 2300 : 1800) * kt + r2);
+    p1.add(units / 2 * p.hkv, item);
+    p1.add(units % 2 * p.hkv, lone);
+    p2.add(n / 2 * p.hq, item);
+    p2.add(n % 2 * p.hq, lone);
+  }
+  constexpr double kStart = 5600;  // attn_persist's, beyond that of the others
+  double best = t2.share(sms);
+  int kernel = 2;
+  *persist = false;
+  const auto offer = [&](double cost, int k, bool persistent) {
+    if (cost >= best) return;
+    best = cost;
+    kernel = k;
+    *persist = persistent;
+  };
+  if (t1.items <= static_cast<long long>(kMaxWaves) * sms) offer(t1.share(sms), 1, false);
+  if (t2.items > sms) offer(kStart + p2.share(sms), 2, true);
+  offer(kStart + p1.share(sms), 1, true);
+  return kernel;
+}
+
 // 1 or 2 (`forced`, or the cheaper one), with whether attn_persist runs it.
 int choose_tc(const AttnParams& p, int sms, int forced, bool* persist) {
   TcEstimate tiles, pairs, group_items, pair_items;
@@ -980,6 +1067,7 @@ int choose_tc(const AttnParams& p, int sms, int forced, bool* persist) {
     pair_items.add(n % 2 * p.hq, 7000.0 + 2000.0 * kt);
   }
   const bool wave1 = tiles.items <= sms, wave2 = pairs.items <= sms;
+  if (forced == 0 && !wave1 && pairs.items <= static_cast<long long>(kMaxWaves) * sms) return few_waves(p, sms, persist);
   const double c1 = wave1 ? tiles.longest : group_items.persistent(sms);
   const double c2 = wave2 ? pairs.longest : pair_items.persistent(sms);
   const int kernel = forced != 0 ? forced : c2 <= c1 ? 2 : 1;
