@@ -488,12 +488,16 @@ __device__ __forceinline__ int finalize_row(const ScoreParams& p, int row, const
   if (write_state) p.state_out[row] = static_cast<uint8_t>(ns);
   if (p.w_out) p.w_out[row] = w;
   if (kExtra && p.p_cur) {
-    p.p_cur[row] = (valid && lc != -INFINITY) ? ex2_approx((lc - a.m) * kLog2e) / z : 0.f;
+    // (one rounding in the exponent; that of m log2 e is taken out as 2^-d = 1 - d ln 2)
+    const float mL = __fmul_rn(a.m, kLog2e), d = fmaf(a.m, kLog2e, -mL);
+    const float e = ex2_approx(fmaf(lc, kLog2e, -mL));
+    p.p_cur[row] = (valid && lc != -INFINITY) ? fmaf(-0.6931471805599453f * d, e, e) / z : 0.f;
   }
   if (kExtra && p.tokens) p.tokens[row] = ns == kStateM ? p.mask_token : a.idx;
   if constexpr (kExtra) {
     // entropy (nats) and margin of the scored distribution, the next step's ordering key
-    const float hnat = valid ? logf(z) + a.m - a.hx / z : 0.f;  // ln Z - (hx - m Z) / Z
+    // ln Z - (hx - m Z) / Z: the two close terms first
+    const float hnat = valid ? (a.m - a.hx / z) + logf(z) : 0.f;
     const float mg = valid ? (1.0f - ex2_approx((a.m2 - a.m) * kLog2e)) / z : 0.f;
     if (p.entropy) p.entropy[row] = hnat;
     if (p.margin) p.margin[row] = mg;
